@@ -59,7 +59,9 @@ typedef enum {
 } submat_status;
 
 typedef enum {
-  SUBMAT_FP64 = 0,               /* Newton-Schulz in FP64 throughout */
+  SUBMAT_FP64 = 0,               /* Newton-Schulz at FP64 accuracy: fixed-point products exact in
+                                    residue arithmetic on the tensor cores (the SIMT GEMM where
+                                    the workspace is too small for them) */
   SUBMAT_FP32 = 1,               /* Newton-Schulz in FP32 (no refinement) */
   SUBMAT_MIXED_BF16_REFINE = 2   /* tensor-core Newton-Schulz on FP16 (hi, lo) pairs, then an
                                     FP64-anchored correction from BF16 and exact sliced
@@ -154,7 +156,7 @@ typedef struct {
    *   (split products and the Lyapunov CG);  2 FP64/FP32 SIMT GEMM;
    *   3 gather (assembly) kernel;  4 tensor-core GEMM, sliced FP64-accurate
    *   residual products;  5 tensor-core GEMM, adjoint (adjoint_mode 1);
-   *   6 extraction (scatter) kernel;  7 reserved.
+   *   6 extraction (scatter) kernel;  7 FP64-accurate residue products.
    * kernel_ms: summed launch durations.  kernel_work: algorithmic work of
    * those launches -- flops for the GEMM classes at the standard count (2 n^3
    * per n x n product the method needs, also where the kernels compute only

@@ -14,6 +14,8 @@
 
 #include "common.cuh"
 #include "plan.cuh"
+#include "rns.cuh"
+#include "tc_gemm.cuh"
 
 namespace submat {
 
@@ -52,6 +54,7 @@ submat_status dev_alloc(void** p, size_t bytes, const char* what) {
 Plan::~Plan() {
   free_mixed(mixed);
   free_adjoint_tc(adj_tc);
+  free_rns(rns);
   for (void* p : owned) cudaFree(p);
   if (h_pinned) cudaFreeHost(h_pinned);
   for (auto& e : ev) if (e) cudaEventDestroy(e);
@@ -452,12 +455,22 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
     }
   }
   // waves
-  const size_t bpe = bytes_per_elem(opt.prec, opt.kT);
+  size_t bpe = bytes_per_elem(opt.prec, opt.kT);
   size_t cap = opt.workspace_cap_bytes;
-  if (cap == 0) {
-    size_t fre = 0, tot = 0;
-    SM_CUDA(cudaMemGetInfo(&fre, &tot));
-    cap = size_t(double(fre) * 0.8);
+  size_t fre = 0, tot = 0;
+  SM_CUDA(cudaMemGetInfo(&fre, &tot));
+  if (cap == 0) cap = size_t(double(fre) * 0.8);
+  if (opt.prec == SUBMAT_FP64 && opt.kT == 0.0) {
+    // residue products (72 B per element) wherever the largest submatrix fits
+    // the workspace that way (21x faster at 420-480 dims, and never slower: one
+    // 64-wide SIMT tile alone takes ~65 us); the SIMT GEMM (24 B) below that
+    const size_t ld = size_t(n_max + 63) / 64 * 64;
+    const size_t room = std::min(cap, size_t(double(fre) * 0.8));
+    use_rns = ld * ld * rns_bytes_per_elem() <= room;
+    if (use_rns) {
+      bpe = rns_bytes_per_elem();
+      cap = room;
+    }
   }
   // the evaluated submatrices (a column range without groups)
   col_lo = opt.col_end > opt.col_begin ? opt.col_begin : 0;
@@ -641,11 +654,118 @@ submat_status Plan::ns_simt(const Wave& wv, T* buf0, T* buf1, T* Y, double tol, 
   return SUBMAT_OK;
 }
 
+// ---------------------------------------------------------------------------
+// FP64 Newton-Schulz by residue products (rns.cuh)
+// ---------------------------------------------------------------------------
+
+long long timeout_cycles_for(double seconds);
+int num_sms();
+
+struct RnsState {
+  std::vector<CUtensorMap*> maps;  // per wave: [residue set][bucket]
+  unsigned* norm2 = nullptr;       // per slot
+};
+
+void free_rns(void* state) { delete static_cast<RnsState*>(state); }
+
+size_t rns_bytes_per_elem() { return 8 + 8 + 2 * 2 * RNS_MODS; }
+
+// Tensor maps of the two residue sets, which follow X and F in the workspace.
+submat_status Plan::rns_setup(cudaStream_t st) {
+  std::unique_ptr<RnsState> r(new RnsState());
+  __nv_bfloat16* base = reinterpret_cast<__nv_bfloat16*>(static_cast<double*>(ws) + 2 * ws_elems);
+  for (auto& wv : waves) {
+    const size_t nbk = wv.bucket_ld.size();
+    std::vector<CUtensorMap> maps(2 * nbk);
+    for (size_t i = 0; i < 2 * nbk; ++i) {
+      const size_t k = i % nbk;
+      const __nv_bfloat16* p = base + RNS_MODS * (int64_t(i / nbk) * ws_elems + wv.bucket_base[k]);
+      if (make_bucket_map(&maps[i], p, int(wv.bucket_ld[k]), wv.bucket_count[k] * RNS_MODS) != 0) {
+        set_error("cuTensorMapEncodeTiled failed");
+        return SUBMAT_ERR_CUDA;
+      }
+    }
+    CUtensorMap* d = nullptr;
+    SM_TRY(put(&d, maps, st, "tensor maps"));
+    SM_CUDA(cudaStreamSynchronize(st));  // the host array goes out of scope
+    r->maps.push_back(d);
+  }
+  SM_TRY(alloc(&r->norm2, size_t(max_wave), "row norms"));
+  rns = r.release();
+  return SUBMAT_OK;
+}
+
+// Newton-Schulz on one wave with X_0 = a / beta in the first buffer, which ends
+// as sign(a).  X moves as 2^-58 fixed point on its upper tiles; a product pass
+// (F on upper 128 x 128 tiles) and a pass over 64 x 64 tile pairs alternate.
+// The first square keeps FP64 and measured operand scales, since rho(X_0) is
+// certified only from it; from then on rho(X) and rho(X^2) are at most 1
+// (1.7146 and 2.94 for X_0, hence its shifts 1 and 2).
+submat_status Plan::ns_rns(size_t wi, cudaStream_t st) {
+  const Wave& wv = waves[wi];
+  auto* r = static_cast<RnsState*>(rns);
+  double* X = static_cast<double*>(ws);
+  long long* F = reinterpret_cast<long long*>(X + ws_elems);
+  __nv_bfloat16* R[2];
+  R[0] = reinterpret_cast<__nv_bfloat16*>(X + 2 * ws_elems);
+  R[1] = R[0] + RNS_MODS * ws_elems;
+  const int nbk = int(wv.bucket_ld.size()), mld = max_ld(wv), nsm = num_sms();
+  const long long tmo = timeout_cycles_for(2.0);
+  auto product = [&](int b) -> submat_status {  // F = X (b = 0: X, 1: Y)
+    RnsGemmParams p{};
+    p.items = wv.sym128; p.nitems = wv.n_sym128;
+    p.map_a = r->maps[wi];
+    p.map_b = r->maps[wi] + b * nbk;
+    p.off = wv.dev.off; p.ld = wv.dev.ld;
+    p.state = ns.state; p.skip_state = ST_DONE;
+    p.split = rns_split(p.nitems, nsm);
+    p.F = F;
+    p.flags = d_flags;
+    p.timeout_cycles = tmo;
+    if (p.split > 1) SM_CUDA(cudaMemsetAsync(F, 0, size_t(wv.elems) * 8, st));
+    size_t tk;
+    SM_TRY(timer.start(KC_RNS, st, &tk));
+    SM_CUDA(launch_rns_gemm(p, nsm, st));
+    SM_TRY(timer.stop(tk, st));
+    return SUBMAT_OK;
+  };
+  for (int k = 0; k < opt.max_iter; ++k) {
+    if (k == 0) {
+      SM_CUDA(launch_rns_rownorm(wv.dev, X, ns.state, r->norm2, mld, st));
+      SM_CUDA(launch_rns_convert(wv.dev, X, ns.state, r->norm2, 0, R[0], nullptr, mld, st));
+      SM_TRY(product(0));
+      SM_CUDA(launch_rns_square0(wv.dev, ns, r->norm2, F, mld, st));
+      if (opt.beta_mode == 0) {  // the power estimate's scale, proven from X_0^2 or reduced
+        const CertSquare sq{0, F, nullptr, 1.0f, 0.0f};
+        const CertLinear lin{1, {X, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
+        SM_CUDA(launch_certify(wv.dev, ns, sq, lin, cert_limits(false), mld, d_flags + 2, st));
+      }
+      SM_CUDA(launch_ns_update(wv.dev, ns, tol_eff, 1e-9, opt.max_iter, d_flags, st));
+      SM_CUDA(launch_rns_convert(wv.dev, X, ns.state, nullptr, 1, R[0], reinterpret_cast<long long*>(X), mld, st));
+      SM_CUDA(launch_rns_convert(wv.dev, reinterpret_cast<double*>(F), ns.state, nullptr, 2, R[1], nullptr, mld, st));
+    } else {
+      SM_TRY(product(0));
+      SM_CUDA(launch_rns_square(wv.dev, ns, F, R[1], mld, st));
+      SM_CUDA(launch_ns_update(wv.dev, ns, tol_eff, 1e-9, opt.max_iter, d_flags, st));
+    }
+    SM_TRY(product(1));
+    SM_CUDA(launch_rns_update(wv.dev, ns, F, k == 0 ? 3 : 0, reinterpret_cast<long long*>(X), R[0], mld, st));
+    SM_CUDA(cudaMemsetAsync(d_active, 0, sizeof(int), st));
+    SM_CUDA(launch_ns_post(wv.dev, ns, 0, d_active, st));
+    SM_CUDA(cudaMemcpyAsync(h_pinned, d_active, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SM_CUDA(cudaStreamSynchronize(st));
+    if (reinterpret_cast<int*>(h_pinned)[0] == 0) break;
+  }
+  return SUBMAT_OK;
+}
+
 submat_status Plan::sign_fp64(const double* K, double mu, double* D, cudaStream_t st) {
   double* B0 = static_cast<double*>(ws);
-  double* B1 = B0 + ws_elems;
-  double* Y = B1 + ws_elems;
-  for (auto& wv : waves) {
+  // residue products leave the result in the first buffer
+  double* B1 = use_rns ? B0 : B0 + ws_elems;
+  if (use_rns && !rns) SM_TRY(rns_setup(st));
+  for (size_t wi = 0; wi < waves.size(); ++wi) {
+    Wave& wv = waves[wi];
     SM_CUDA(cudaEventRecord(ev[0], st));
     SM_TRY(gather_wave(wv, K, mu, B0, st));
     SM_CUDA(launch_scale_f64(wv.dev, B0, B0, ns.beta, wv.max_ld2, st));
@@ -655,8 +775,12 @@ submat_status Plan::sign_fp64(const double* K, double mu, double* D, cudaStream_
       SM_CUDA(launch_reset_rprev(wv.dev, ns, st));
     }
     SM_CUDA(cudaEventRecord(ev[1], st));
-    SM_TRY((ns_simt<double, GemmF64Args>(wv, B0, B1, Y, tol_eff, 1e-9, st, launch_gemm_f64,
-                                         opt.beta_mode == 0)));
+    if (use_rns) {
+      SM_TRY(ns_rns(wi, st));
+    } else {
+      SM_TRY((ns_simt<double, GemmF64Args>(wv, B0, B1, B1 + ws_elems, tol_eff, 1e-9, st, launch_gemm_f64,
+                                           opt.beta_mode == 0)));
+    }
     SM_CUDA(cudaEventRecord(ev[2], st));
     SM_TRY(scatter_timed(wv, 16.0, [&] { return launch_scatter_f64(g, wv.dev, ns, B0, B1, D, d_trpart, geom(wv), st); },
                          st));
@@ -769,7 +893,7 @@ void Plan::finish_stats(bool adjoint) {
       // two products per iteration, 2 n^3 flops each at the standard count
       for (int j = col_lo; j < col_hi; ++j) {
         const double n = qn[j];
-        stats.kernel_work[KC_SIMT] += 4.0 * n * n * n * res_iters[j];
+        stats.kernel_work[use_rns ? KC_RNS : KC_SIMT] += 4.0 * n * n * n * res_iters[j];
       }
     }
   }

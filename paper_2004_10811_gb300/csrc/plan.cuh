@@ -21,6 +21,8 @@ constexpr int kPowerIters = 10;  // power steps of the spectral estimate
 constexpr int kProbeMaxIter = 40;  // Newton-Schulz cap of a mu-search probe
 void free_mixed(void* state);
 void free_adjoint_tc(void* state);
+void free_rns(void* state);
+size_t rns_bytes_per_elem();  // FP64 path by residue products: X, F and two residue sets
 
 // Launch plan of an exact sliced product (mixed.cu).  Slices are numbered
 // 1..n; a group is one exact accumulator: np products (pr[i] = (p, q)) of one
@@ -130,6 +132,7 @@ struct KernelTimer {
 
 enum KernelClass {
   KC_TC_NS = 0, KC_TC_REF = 1, KC_SIMT = 2, KC_GATHER = 3, KC_TC_HP = 4, KC_TC_ADJ = 5, KC_SCATTER = 6,
+  KC_RNS = 7,
   KC_COUNT = 8
 };
 
@@ -181,6 +184,8 @@ struct Plan {
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   std::vector<void*> owned;
   void* mixed = nullptr;       // mixed-path state (mixed.cu)
+  void* rns = nullptr;         // residue-product state of the FP64 path (plan.cu); null: SIMT GEMM
+  bool use_rns = false;
   void* adj_tc = nullptr;      // tensor-core adjoint state (mixed.cu)
   // adjoint: its own waves and workspace (six dense buffers per submatrix)
   std::vector<Wave> bwaves;
@@ -256,6 +261,8 @@ struct Plan {
   submat_status backward_wave_tc(size_t wi, const double* K, double mu, const double* Dbar, double* Kbar,
                                  double* dn_part, cudaStream_t st);
   submat_status grow_ns_state(int count);
+  submat_status rns_setup(cudaStream_t st);
+  submat_status ns_rns(size_t wi, cudaStream_t st);
   template <typename T, typename Args>
   submat_status ns_simt(const Wave& wv, T* buf0, T* buf1, T* Y, double tol, double floor_thr,
                         cudaStream_t st, cudaError_t (*gemm)(const Args&, cudaStream_t), bool certify);
