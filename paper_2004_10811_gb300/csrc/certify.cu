@@ -67,10 +67,23 @@ __global__ void __launch_bounds__(256) k_cert_rowsum(WaveDev w, CertSquare sq, c
       }
     } else if (sq.mode == 1) {
       const float* x = static_cast<const float*>(sq.hi);
-      for (int c = lane; c < ld; c += 32) acc += fabsf(x[row + c]);
+      // at alpha = 2 never below q's own row sum, which has been the scale of
+      // FP32 series all along (a larger scale is safe; theirs stays put)
+      float own = 0.0f;
+      for (int c = lane; c < ld; c += 32) {
+        own += fabsf(x[row + c]);
+        acc += fabsf((x[row + c] - (c == r ? sq.diag : 0.0f)) * ia);
+      }
+      double t = double(own);
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      best = fmax(best, t);
     } else {
       const double* x = static_cast<const double*>(sq.hi);
-      for (int c = lane; c < ld; c += 32) acc += fabsf(float(x[row + c]));
+      for (int c = lane; c < ld; c += 32) {
+        double v = x[row + c];
+        if (c == r) v -= double(sq.diag);
+        acc += fabsf(float(v) * ia);
+      }
     }
     double t = double(acc);
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);

@@ -175,8 +175,8 @@ cudaError_t launch_rescale_f32(const WaveDev& w, float* X, const double* rho, do
 // After the first squaring, ||X_0^2||_inf >= rho(X_0)^2 proves that the power
 // estimate's scale keeps the spectrum of X_0 inside the iteration's basin;
 // where it cannot, X_0 (and everything derived from it) is scaled down.
-// Representation of the squared iterate: 0 FP64 X^2, 1 FP32 X^2, 2 a BF16
-// (hi, lo) pair holding q = diag I + alpha X^2.
+// Representation of the squared iterate q = diag I + alpha X^2: 0 FP64, 1 FP32,
+// 2 a BF16 (hi, lo) pair.
 struct CertSquare {
   int mode;        // 0 FP64, 1 FP32, 2 BF16 (hi, lo) pair, 3 FP16 pair
   void* hi;        // the square (FP64 / FP32 array, or the pair's hi)

@@ -239,3 +239,16 @@ def test_band_energy_gradient_matches_central_differences(pkg):
             fd = (vals[0] - vals[1]) / (2 * h)
             an = grad[p] + (grad[q] if q != p else 0.0)
             assert abs(an - fd) <= 1e-6 * max(1.0, abs(fd)), (p, an, fd)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_scale_bounds_the_spectrum(pkg, prec):
+    """a = x [[1, 1], [1, -1]]: (a / beta)^2 = I / 2 exactly, where 2 X^2 - I is 0
+    and says nothing about rho(X) = 1 / sqrt 2."""
+    from synth.water import BSRMatrix
+    for x in (0.6, 0.011):
+        m = BSRMatrix(np.array([2], np.int32), np.array([0, 1]), np.array([0], np.int32),
+                      x * np.array([1.0, 1.0, 1.0, -1.0]))
+        got, _tr, st = run(pkg, m, 0.0, 0.1, prec=prec)
+        assert float(np.max(np.abs(got - oracle.density_matrix_T(m, 0.0, 0.1)))) <= (1e-12 if prec == "fp64" else 2e-6)
+        assert st["poly_degree"] >= 3
