@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "plan.cuh"
+#include "rns.cuh"
 
 namespace submat {
 
@@ -123,6 +124,29 @@ submat_status fermi_poly(double c, double tol, int max_degree, FermiPoly* out) {
     }
   for (int i = 1; i < S; i += 2) P.r[i / 2] = a[i];
   return SUBMAT_OK;
+}
+
+int fermi_clenshaw_exponent(const FermiPoly& P) {
+  // The terms are polynomials of degree m or less: their maximum on [-1, 1] is
+  // at most 1 / cos(pi / 4) times that over 2 (m + 1) Chebyshev nodes (Ehlich
+  // and Zeller 1964).  They are odd or even, so half of the nodes suffice.
+  constexpr int H = kFermiBaby / 2;
+  const int nodes = 2 * (P.m + 1);
+  double mx = 0.0;
+  for (int i = 0; 2 * i < nodes; ++i) {
+    const double th = M_PI * (2 * i + 1) / (2.0 * nodes), y = std::cos(kFermiBaby * th);
+    double t[H], b1 = 0.0, b2 = 0.0;
+    for (int q = 0; q < H; ++q) t[q] = std::cos((2 * q + 1) * th);
+    for (int j = P.blocks - 1; j >= 0; --j) {
+      double R = 0.0;
+      for (int q = 0; q < H; ++q) R += P.r[size_t(j) * H + q] * t[q];
+      const double b = R + (j == 0 ? 1.0 : 2.0) * y * b1 - b2;  // at j = 0: p
+      mx = std::max(mx, std::fabs(b));
+      b2 = b1;
+      b1 = b;
+    }
+  }
+  return std::max(0, int(std::ceil(std::log2(std::max(1e-300, 1.4143 * mx)))));
 }
 
 namespace {
@@ -225,7 +249,7 @@ size_t fermi_dual_bytes_per_elem(int prec) {
 // came from (L_f(a, .) is self-adjoint in the Frobenius product for
 // symmetric a).  The value part is evaluated exactly as in the forward path.
 template <typename T>
-submat_status Plan::fermi_wave(Wave& wv, const double* K, double mu, double* D, const double* Dbar, double* Kbar,
+submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, double* D, const double* Dbar, double* Kbar,
                                void* w, int64_t E, cudaStream_t st) {
   using G = FermiGemm<T>;
   using Args = typename G::Args;
@@ -277,7 +301,17 @@ submat_status Plan::fermi_wave(Wave& wv, const double* K, double mu, double* D, 
     return SUBMAT_OK;
   };
   // T_2 = 2 X^2 - I at X = a / beta_bound, and from it the tight scale
-  SM_TRY(gemm(odd, odd, nullptr, T2, 2.0, 0.0, -1.0));
+  const bool residues = wi >= 0;  // FP64 forward only
+  if (residues) {
+    long long* F = reinterpret_cast<long long*>(A);  // A has served its purpose
+    SM_CUDA(launch_rns_convert(wv.dev, reinterpret_cast<double*>(odd), nullptr, nullptr, 0, rns_residues(1), nullptr,
+                               max_ld(wv), st));
+    SM_TRY(rns_product(size_t(wi), 1, 1, F, nullptr, st));
+    SM_CUDA(launch_rns_cheb2(wv.dev, F, reinterpret_cast<double*>(T2), max_ld(wv), st));
+    ++products;
+  } else {
+    SM_TRY(gemm(odd, odd, nullptr, T2, 2.0, 0.0, -1.0));
+  }
   const CertSquare sq{f64 ? 0 : 1, T2, nullptr, 2.0f, -1.0f};
   SM_CUDA(cudaMemsetAsync(ns.cert, 0, sizeof(unsigned long long) * wv.count, st));
   SM_CUDA(launch_cert_rowsum(wv.dev, ns, sq, max_ld(wv), st));
@@ -320,41 +354,47 @@ submat_status Plan::fermi_wave(Wave& wv, const double* K, double mu, double* D, 
   SM_TRY(fermi_poly(sigma / (2.0 * opt.kT), tol_poly, kFermiMaxDegree, &P));
   fermi_degree = std::max(fermi_degree, P.m);
   fermi_trunc = std::max(fermi_trunc, P.trunc);
-  // baby steps: T_3 = 2 T_2 X - X, T_{k+2} = 2 T_2 T_k - T_{k-2}
-  for (int q = 1; q < S / 2; ++q)
-    SM_TRY(gemm(T2, odd + int64_t(q - 1) * E, q >= 2 ? odd + int64_t(q - 2) * E : odd, odd + int64_t(q) * E,
-                2.0, -1.0, 0.0));
-  // Y = T_16 = 2 T_9 T_7 - T_2, in T_2's buffer
-  SM_TRY(gemm(odd + 4 * E, odd + 3 * E, T2, T2, 2.0, -1.0, 0.0));
-  const T* Y = T2;
-  // giant steps: Clenshaw in Y with the coefficients R_j
-  auto comb = [&](int j, const T* B, T* W) -> submat_status {
-    CombArgs ca;
-    for (int q = 0; q < S / 2; ++q) ca.r[q] = P.r[size_t(j) * (S / 2) + q];
-    k_cheb_comb<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, odd, E, ca, B, W);
-    SM_KCHECK();
-    if (dual) {
-      k_cheb_comb<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, dp(odd), E, ca, dp(B), dp(W));
-      SM_KCHECK();
-    }
-    return SUBMAT_OK;
-  };
   T* out = nullptr;
-  if (P.blocks == 1) {
-    SM_TRY(comb(0, nullptr, bb[0]));
-    out = bb[0];
+  if (residues) {
+    double* o = nullptr;
+    SM_TRY(fermi_rns(wi, P, &o, &products, st));
+    out = reinterpret_cast<T*>(o);
   } else {
-    T* b1 = bb[0];     // b_{j+1}
-    T* b2 = nullptr;   // b_{j+2} (b_G = 0 at the start)
-    SM_TRY(comb(P.blocks - 1, nullptr, b1));
-    for (int j = P.blocks - 2; j >= 0; --j) {
-      // W = R_j - b_{j+2} (in place over b_{j+2}), then W += c Y b_{j+1}
-      T* W = b2 ? b2 : bb[1];
-      SM_TRY(comb(j, b2, W));
-      SM_TRY(gemm(Y, b1, W, W, j == 0 ? 1.0 : 2.0, 1.0, 0.0));
-      if (j == 0) { out = W; break; }
-      b2 = b1;
-      b1 = W;
+    // baby steps: T_3 = 2 T_2 X - X, T_{k+2} = 2 T_2 T_k - T_{k-2}
+    for (int q = 1; q < S / 2; ++q)
+      SM_TRY(gemm(T2, odd + int64_t(q - 1) * E, q >= 2 ? odd + int64_t(q - 2) * E : odd, odd + int64_t(q) * E,
+                  2.0, -1.0, 0.0));
+    // Y = T_16 = 2 T_9 T_7 - T_2, in T_2's buffer
+    SM_TRY(gemm(odd + 4 * E, odd + 3 * E, T2, T2, 2.0, -1.0, 0.0));
+    const T* Y = T2;
+    // giant steps: Clenshaw in Y with the coefficients R_j
+    auto comb = [&](int j, const T* B, T* W) -> submat_status {
+      CombArgs ca;
+      for (int q = 0; q < S / 2; ++q) ca.r[q] = P.r[size_t(j) * (S / 2) + q];
+      k_cheb_comb<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, odd, E, ca, B, W);
+      SM_KCHECK();
+      if (dual) {
+        k_cheb_comb<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, dp(odd), E, ca, dp(B), dp(W));
+        SM_KCHECK();
+      }
+      return SUBMAT_OK;
+    };
+    if (P.blocks == 1) {
+      SM_TRY(comb(0, nullptr, bb[0]));
+      out = bb[0];
+    } else {
+      T* b1 = bb[0];     // b_{j+1}
+      T* b2 = nullptr;   // b_{j+2} (b_G = 0 at the start)
+      SM_TRY(comb(P.blocks - 1, nullptr, b1));
+      for (int j = P.blocks - 2; j >= 0; --j) {
+        // W = R_j - b_{j+2} (in place over b_{j+2}), then W += c Y b_{j+1}
+        T* W = b2 ? b2 : bb[1];
+        SM_TRY(comb(j, b2, W));
+        SM_TRY(gemm(Y, b1, W, W, j == 0 ? 1.0 : 2.0, 1.0, 0.0));
+        if (j == 0) { out = W; break; }
+        b2 = b1;
+        b1 = W;
+      }
     }
   }
   SM_CUDA(cudaEventRecord(ev[2], st));
@@ -374,9 +414,84 @@ submat_status Plan::fermi_wave(Wave& wv, const double* K, double mu, double* D, 
   return SUBMAT_OK;
 }
 
+// The recurrences of fermi_wave on exact residue products (rns.cuh), from X
+// and T_2 in FP64.  Every T_k has norm 1 or less; the Clenshaw terms move as
+// b_j 2^-e (fermi_clenshaw_exponent).  Residue set 0 holds the factor that
+// stays (T_2, then Y), set 1 the one that each pass renews.
+// 720 submatrices of 240 molecules (13 + 5 + 5 functions, 6.5 A, kT 0.05): a
+// build took 573 ms with the FP64 SIMT GEMM and takes 28.3 ms.
+submat_status Plan::fermi_rns(int wi, const FermiPoly& P, double** out, int* products, cudaStream_t st) {
+  constexpr int H = kFermiBaby / 2;
+  static_assert(H == RNS_COMB, "one coefficient per stored odd T_k");
+  const Wave& wv = waves[size_t(wi)];
+  const int64_t E = ws_elems;
+  const int mld = max_ld(wv), e = fermi_clenshaw_exponent(P);
+  long long* F = static_cast<long long*>(ws);
+  long long* odd = F + E;
+  long long* T2 = odd + H * E;
+  long long* bb[2] = {T2 + E, T2 + 2 * E};
+  __nv_bfloat16* R[2] = {rns_residues(0), rns_residues(1)};
+  auto product = [&]() -> submat_status {  // F = (set 0) (set 1)
+    ++*products;
+    return rns_product(size_t(wi), 0, 1, F, nullptr, st);
+  };
+  auto dbl = [](long long* p) { return reinterpret_cast<double*>(p); };
+  SM_CUDA(launch_rns_convert(wv.dev, dbl(odd), nullptr, nullptr, 0, R[1], odd, mld, st));
+  SM_CUDA(launch_rns_convert(wv.dev, dbl(T2), nullptr, nullptr, 0, R[0], T2, mld, st));
+  RnsCheb c{};
+  c.F = F;
+  c.twice = 1;
+  c.R = R[1];
+  for (int q = 1; q < H; ++q) {  // T_{2q+1} = 2 T_2 T_{2q-1} - T_{2q-3}, T_{-1} = T_1
+    SM_TRY(product());
+    c.sub = odd + int64_t(std::max(0, q - 2)) * E;
+    c.C = odd + int64_t(q) * E;
+    if (q == H - 1) c.R = nullptr;
+    SM_CUDA(launch_rns_cheb(wv.dev, c, mld, st));
+  }
+  for (int i = 0; i < 2; ++i) {  // residues of -T_9 and -T_7
+    RnsCheb t{};
+    t.sub = odd + int64_t(H / 2 - i) * E;
+    t.R = R[i];
+    SM_CUDA(launch_rns_cheb(wv.dev, t, mld, st));
+  }
+  SM_TRY(product());  // Y = T_16 = 2 T_9 T_7 - T_2
+  c.sub = T2;
+  c.C = T2;
+  c.R = R[0];
+  SM_CUDA(launch_rns_cheb(wv.dev, c, mld, st));
+  // giant steps: b_j = R_j + 2 Y b_{j+1} - b_{j+2}, p = R_0 + Y b_1 - b_2
+  c = RnsCheb{};
+  c.odd = odd;
+  c.stride = E;
+  c.R = R[1];
+  for (int j = P.blocks - 1; j >= 0; --j) {
+    long long* W = bb[j & 1];  // b_{j+2}'s place
+    for (int q = 0; q < H; ++q) c.coef[q] = std::llrint(std::ldexp(P.r[size_t(j) * H + q], 60 - e));
+    if (j < P.blocks - 1) {
+      SM_TRY(product());
+      c.F = F;
+    }
+    c.twice = j > 0;
+    c.sub = j < P.blocks - 2 ? W : nullptr;
+    c.C = W;
+    if (j == 0) {
+      c.C = nullptr;
+      c.R = nullptr;
+      c.out = dbl(W);
+      c.out_scale = std::ldexp(1.0, e - RNS_FRAC);
+      *out = c.out;
+    }
+    SM_CUDA(launch_rns_cheb(wv.dev, c, mld, st));
+  }
+  return SUBMAT_OK;
+}
+
 template <typename T>
 submat_status Plan::sign_fermi(const double* K, double mu, double* D, cudaStream_t st) {
-  for (auto& wv : waves) SM_TRY(fermi_wave<T>(wv, K, mu, D, nullptr, nullptr, ws, ws_elems, st));
+  if (use_rns && !rns) SM_TRY(rns_setup(st));
+  for (size_t wi = 0; wi < waves.size(); ++wi)
+    SM_TRY(fermi_wave<T>(waves[wi], use_rns ? int(wi) : -1, K, mu, D, nullptr, nullptr, ws, ws_elems, st));
   return SUBMAT_OK;
 }
 
@@ -434,8 +549,8 @@ submat_status Plan::backward_fermi(const double* K, double mu, const double* Dba
   }
   SM_CUDA(cudaMemsetAsync(Kbar, 0, sizeof(double) * size_t(nvals), st));
   for (auto& wv : bwaves) {
-    if (opt.prec == SUBMAT_FP64) SM_TRY(fermi_wave<double>(wv, K, mu, nullptr, Dbar, Kbar, bws, bws_elems, st));
-    else SM_TRY(fermi_wave<float>(wv, K, mu, nullptr, Dbar, Kbar, bws, bws_elems, st));
+    if (opt.prec == SUBMAT_FP64) SM_TRY(fermi_wave<double>(wv, -1, K, mu, nullptr, Dbar, Kbar, bws, bws_elems, st));
+    else SM_TRY(fermi_wave<float>(wv, -1, K, mu, nullptr, Dbar, Kbar, bws, bws_elems, st));
   }
   SM_CUDA(cudaStreamSynchronize(st));
   finish_stats(true);

@@ -460,15 +460,16 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
   size_t fre = 0, tot = 0;
   SM_CUDA(cudaMemGetInfo(&fre, &tot));
   if (cap == 0) cap = size_t(double(fre) * 0.8);
-  if (opt.prec == SUBMAT_FP64 && opt.kT == 0.0) {
-    // residue products (72 B per element) wherever the largest submatrix fits
-    // the workspace that way (21x faster at 420-480 dims, and never slower: one
-    // 64-wide SIMT tile alone takes ~65 us); the SIMT GEMM (24 B) below that
+  if (opt.prec == SUBMAT_FP64) {
+    // residue products (72 B per element, 152 B at finite temperature) wherever
+    // the largest submatrix fits the workspace that way (21x faster at 420-480
+    // dims, and never slower: one 64-wide SIMT tile alone takes ~65 us); the
+    // SIMT GEMM (24 B and 96 B) below that
     const size_t ld = size_t(n_max + 63) / 64 * 64;
     const size_t room = std::min(cap, size_t(double(fre) * 0.8));
-    use_rns = ld * ld * rns_bytes_per_elem() <= room;
+    use_rns = ld * ld * (rns_state_bytes() + rns_residue_bytes()) <= room;
     if (use_rns) {
-      bpe = rns_bytes_per_elem();
+      bpe = rns_state_bytes() + rns_residue_bytes();
       cap = room;
     }
   }
@@ -658,9 +659,6 @@ submat_status Plan::ns_simt(const Wave& wv, T* buf0, T* buf1, T* Y, double tol, 
 // FP64 Newton-Schulz by residue products (rns.cuh)
 // ---------------------------------------------------------------------------
 
-long long timeout_cycles_for(double seconds);
-int num_sms();
-
 struct RnsState {
   std::vector<CUtensorMap*> maps;  // per wave: [residue set][bucket]
   unsigned* norm2 = nullptr;       // per slot
@@ -668,12 +666,20 @@ struct RnsState {
 
 void free_rns(void* state) { delete static_cast<RnsState*>(state); }
 
-size_t rns_bytes_per_elem() { return 8 + 8 + 2 * 2 * RNS_MODS; }
+// Bytes per dense element: the matrices that precede the residue sets in the
+// workspace (X and F, or the buffers of fermi_wave), and the two sets.
+size_t Plan::rns_state_bytes() const { return opt.kT > 0.0 ? fermi_bytes_per_elem(SUBMAT_FP64) : 16; }
+size_t rns_residue_bytes() { return 2 * 2 * RNS_MODS; }
 
-// Tensor maps of the two residue sets, which follow X and F in the workspace.
+__nv_bfloat16* Plan::rns_residues(int set) const {
+  return reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(ws) + rns_state_bytes() * size_t(ws_elems)) +
+         int64_t(set) * RNS_MODS * ws_elems;
+}
+
+// Tensor maps of the two residue sets.
 submat_status Plan::rns_setup(cudaStream_t st) {
   std::unique_ptr<RnsState> r(new RnsState());
-  __nv_bfloat16* base = reinterpret_cast<__nv_bfloat16*>(static_cast<double*>(ws) + 2 * ws_elems);
+  __nv_bfloat16* base = rns_residues(0);
   for (auto& wv : waves) {
     const size_t nbk = wv.bucket_ld.size();
     std::vector<CUtensorMap> maps(2 * nbk);
@@ -695,6 +701,31 @@ submat_status Plan::rns_setup(cudaStream_t st) {
   return SUBMAT_OK;
 }
 
+// F = frac of the symmetric product of two residue sets on the upper tiles of a
+// wave; submatrices with state ST_DONE are skipped.
+submat_status Plan::rns_product(size_t wi, int a, int b, long long* F, const int* state, cudaStream_t st) {
+  const Wave& wv = waves[wi];
+  const size_t nbk = wv.bucket_ld.size();
+  const int nsm = num_sms();
+  CUtensorMap* maps = static_cast<const RnsState*>(rns)->maps[wi];
+  RnsGemmParams p{};
+  p.items = wv.sym128; p.nitems = wv.n_sym128;
+  p.map_a = maps + size_t(a) * nbk;
+  p.map_b = maps + size_t(b) * nbk;
+  p.off = wv.dev.off; p.ld = wv.dev.ld;
+  p.state = state; p.skip_state = ST_DONE;
+  p.split = rns_split(p.nitems, nsm);
+  p.F = F;
+  p.flags = d_flags;
+  p.timeout_cycles = kWaitCycles;
+  if (p.split > 1) SM_CUDA(cudaMemsetAsync(F, 0, size_t(wv.elems) * 8, st));
+  size_t tk;
+  SM_TRY(timer.start(KC_RNS, st, &tk));
+  SM_CUDA(launch_rns_gemm(p, nsm, st));
+  SM_TRY(timer.stop(tk, st));
+  return SUBMAT_OK;
+}
+
 // Newton-Schulz on one wave with X_0 = a / beta in the first buffer, which ends
 // as sign(a).  X moves as 2^-58 fixed point on its upper tiles; a product pass
 // (F on upper 128 x 128 tiles) and a pass over 64 x 64 tile pairs alternate.
@@ -706,29 +737,9 @@ submat_status Plan::ns_rns(size_t wi, cudaStream_t st) {
   auto* r = static_cast<RnsState*>(rns);
   double* X = static_cast<double*>(ws);
   long long* F = reinterpret_cast<long long*>(X + ws_elems);
-  __nv_bfloat16* R[2];
-  R[0] = reinterpret_cast<__nv_bfloat16*>(X + 2 * ws_elems);
-  R[1] = R[0] + RNS_MODS * ws_elems;
-  const int nbk = int(wv.bucket_ld.size()), mld = max_ld(wv), nsm = num_sms();
-  const long long tmo = timeout_cycles_for(2.0);
-  auto product = [&](int b) -> submat_status {  // F = X (b = 0: X, 1: Y)
-    RnsGemmParams p{};
-    p.items = wv.sym128; p.nitems = wv.n_sym128;
-    p.map_a = r->maps[wi];
-    p.map_b = r->maps[wi] + b * nbk;
-    p.off = wv.dev.off; p.ld = wv.dev.ld;
-    p.state = ns.state; p.skip_state = ST_DONE;
-    p.split = rns_split(p.nitems, nsm);
-    p.F = F;
-    p.flags = d_flags;
-    p.timeout_cycles = tmo;
-    if (p.split > 1) SM_CUDA(cudaMemsetAsync(F, 0, size_t(wv.elems) * 8, st));
-    size_t tk;
-    SM_TRY(timer.start(KC_RNS, st, &tk));
-    SM_CUDA(launch_rns_gemm(p, nsm, st));
-    SM_TRY(timer.stop(tk, st));
-    return SUBMAT_OK;
-  };
+  __nv_bfloat16* R[2] = {rns_residues(0), rns_residues(1)};
+  const int mld = max_ld(wv);
+  auto product = [&](int b) { return rns_product(wi, 0, b, F, ns.state, st); };  // F = X (b = 0: X, 1: Y)
   for (int k = 0; k < opt.max_iter; ++k) {
     if (k == 0) {
       SM_CUDA(launch_rns_rownorm(wv.dev, X, ns.state, r->norm2, mld, st));
@@ -888,7 +899,7 @@ void Plan::finish_stats(bool adjoint) {
     if (adjoint) {  // every adjoint product runs on one GEMM kind
       stats.kernel_work[opt.adjoint_mode == 1 && opt.kT == 0.0 ? KC_TC_ADJ : KC_SIMT] += flops;
     } else if (opt.kT > 0.0) {
-      stats.kernel_work[KC_SIMT] += flops;
+      stats.kernel_work[use_rns ? KC_RNS : KC_SIMT] += flops;
     } else if (opt.prec != SUBMAT_MIXED_BF16_REFINE) {
       // two products per iteration, 2 n^3 flops each at the standard count
       for (int j = col_lo; j < col_hi; ++j) {

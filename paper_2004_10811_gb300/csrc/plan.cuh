@@ -17,12 +17,16 @@ submat_status validate_pattern_public(int nblk, const int32_t* bs, const int64_t
 const char* last_error();
 size_t mixed_bytes_per_elem();
 size_t adjoint_tc_bytes_per_elem();
+int num_sms();
+// limit of the kernels' bounded waits: 2 s at the GB300's 2.07 GHz, longer at a
+// lower clock (asking the driver for the clock takes 0.6 ms a call)
+constexpr long long kWaitCycles = 4140000000ll;
 constexpr int kPowerIters = 10;  // power steps of the spectral estimate
 constexpr int kProbeMaxIter = 40;  // Newton-Schulz cap of a mu-search probe
 void free_mixed(void* state);
 void free_adjoint_tc(void* state);
 void free_rns(void* state);
-size_t rns_bytes_per_elem();  // FP64 path by residue products: X, F and two residue sets
+size_t rns_residue_bytes();  // the two residue sets of the FP64 path, per dense element
 
 // Launch plan of an exact sliced product (mixed.cu).  Slices are numbered
 // 1..n; a group is one exact accumulator: np products (pr[i] = (p, q)) of one
@@ -70,6 +74,9 @@ struct FermiPoly {
   double trunc = 0.0;  // sum of |c_k| beyond m: bounds the truncation error on [-1, 1]
   std::vector<double> r;
 };
+// Exponent e with |b_j(x)| <= 2^e on [-1, 1] for every Clenshaw term b_j of P
+// and p, 0 at least.
+int fermi_clenshaw_exponent(const FermiPoly& P);
 submat_status fermi_poly(double c, double tol, int max_degree, FermiPoly* out);
 size_t fermi_bytes_per_elem(int prec);
 
@@ -244,10 +251,10 @@ struct Plan {
   template <typename T>
   submat_status sign_fermi(const double* K, double mu, double* D, cudaStream_t st);
   // one wave of the finite-temperature evaluation on workspace `w` of E
-  // elements per buffer; with Dbar set, the polynomial runs on dual numbers
+  // elements per buffer, wi its index for residue products (-1: SIMT); with Dbar set, the polynomial runs on dual numbers
   // and -1/2 of its derivative part (L_f(a_j, G_j)) is added into Kbar
   template <typename T>
-  submat_status fermi_wave(Wave& wv, const double* K, double mu, double* D, const double* Dbar, double* Kbar,
+  submat_status fermi_wave(Wave& wv, int wi, const double* K, double mu, double* D, const double* Dbar, double* Kbar,
                            void* w, int64_t E, cudaStream_t st);
   submat_status fermi_dn_dmu(cudaStream_t st, double* out);
   submat_status backward_fermi(const double* K, double mu, const double* Dbar, double* Kbar, double* dN_dmu,
@@ -262,6 +269,10 @@ struct Plan {
                                  double* dn_part, cudaStream_t st);
   submat_status grow_ns_state(int count);
   submat_status rns_setup(cudaStream_t st);
+  size_t rns_state_bytes() const;
+  __nv_bfloat16* rns_residues(int set) const;
+  submat_status rns_product(size_t wi, int a, int b, long long* F, const int* state, cudaStream_t st);
+  submat_status fermi_rns(int wi, const FermiPoly& P, double** out, int* products, cudaStream_t st);
   submat_status ns_rns(size_t wi, cudaStream_t st);
   template <typename T, typename Args>
   submat_status ns_simt(const Wave& wv, T* buf0, T* buf1, T* Y, double tol, double floor_thr,

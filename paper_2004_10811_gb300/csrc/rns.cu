@@ -625,6 +625,83 @@ __global__ void __launch_bounds__(256) k_rns_update(WaveDev w, NsStateDev ns, co
   }
 }
 
+__global__ void __launch_bounds__(256) k_rns_cheb2(WaveDev w, const long long* __restrict__ F,
+                                                   double* __restrict__ T2) {
+  __shared__ long long v[64][PITCH];
+  const int s = blockIdx.y;
+  const int ld = w.ld[s], n = w.n[s], T = ld / 64;
+  const int64_t base = w.off[s];
+  const int c = (threadIdx.x & 31) * 2;
+  for (int pi = blockIdx.x; pi < T * (T + 1) / 2; pi += gridDim.x) {
+    int a, b;
+    pair_of(pi, T, &a, &b);
+    __syncthreads();
+    for (int r = threadIdx.x >> 5; r < 64; r += 8) {
+      const longlong2 f = *reinterpret_cast<const longlong2*>(F + base + int64_t(a * 64 + r) * ld + b * 64 + c);
+      const bool row = a == b && a * 64 + r < n;  // 2 X^2 - I at 2^-61
+      v[r][c] = product62(f.x) - (row && r == c ? 1ll << 61 : 0);
+      v[r][c + 1] = product62(f.y) - (row && r == c + 1 ? 1ll << 61 : 0);
+    }
+    __syncthreads();
+    tile_doubles(v, a, b, ld, 0x1p-61, T2 + base);
+  }
+}
+
+// One step of the recurrences, as a pass over tile pairs: bound by memory
+// traffic (the residues written, 28 bytes an entry, are the largest part), so
+// the combination of the stored odd T_k is formed here instead of in a pass of
+// its own, and only upper tiles are read.  Its 64-bit upper halves are floors:
+// RNS_COMB / 2 restores their mean (where they are floors of anything but 0).
+template <bool COMB>
+__global__ void __launch_bounds__(256) k_rns_cheb(WaveDev w, const __grid_constant__ RnsCheb p) {
+  __shared__ long long v[64][PITCH];
+  const int s = blockIdx.y;
+  const int ld = w.ld[s], T = ld / 64;
+  const int64_t base = w.off[s], plane = int64_t(ld) * ld;
+  const int c = (threadIdx.x & 31) * 2;
+  const int sh = p.twice ? 3 : 4;  // product62 to 2^-58
+  for (int pi = blockIdx.x; pi < T * (T + 1) / 2; pi += gridDim.x) {
+    int a, b;
+    pair_of(pi, T, &a, &b);
+    __syncthreads();
+#pragma unroll 2
+    for (int r = threadIdx.x >> 5; r < 64; r += 8) {
+      const int64_t i = base + int64_t(a * 64 + r) * ld + b * 64 + c;
+      longlong2 x = make_longlong2(0, 0);
+      if (p.F) {
+        const longlong2 f = *reinterpret_cast<const longlong2*>(p.F + i);
+        const long long half = (1ll << sh) >> 1;
+        x.x = (product62(f.x) + half) >> sh;
+        x.y = (product62(f.y) + half) >> sh;
+      }
+      if (p.sub) {
+        const longlong2 z = *reinterpret_cast<const longlong2*>(p.sub + i);
+        x.x -= z.x;
+        x.y -= z.y;
+      }
+      if constexpr (COMB) {
+        longlong2 any = make_longlong2(0, 0);
+#pragma unroll
+        for (int q = 0; q < RNS_COMB; ++q) {
+          const longlong2 t = *reinterpret_cast<const longlong2*>(p.odd + q * p.stride + i);
+          x.x += __mul64hi(t.x << 4, p.coef[q]);  // 2^-62 2^-60 2^64
+          x.y += __mul64hi(t.y << 4, p.coef[q]);
+          any.x |= t.x;
+          any.y |= t.y;
+        }
+        x.x += any.x ? RNS_COMB / 2 : 0;
+        x.y += any.y ? RNS_COMB / 2 : 0;
+      }
+      v[r][c] = x.x;
+      v[r][c + 1] = x.y;
+      if (p.C) *reinterpret_cast<longlong2*>(p.C + i) = x;
+    }
+    __syncthreads();
+    if (p.out) tile_doubles(v, a, b, ld, p.out_scale, p.out + base);
+    if (p.R) tile_residues(v, a, b, ld, p.R + RNS_MODS * base, plane);
+  }
+}
+
 // about four tile pairs a block
 dim3 tile_grid(int max_ld, int nsub) {
   const int T = max_ld / 64;
@@ -685,6 +762,19 @@ cudaError_t launch_rns_square(const WaveDev& w, NsStateDev ns, const long long* 
 cudaError_t launch_rns_update(const WaveDev& w, NsStateDev ns, const long long* F, int shift, long long* X,
                               __nv_bfloat16* R, int max_ld, cudaStream_t st) {
   k_rns_update<<<tile_grid(max_ld, w.nsub), 256, 0, st>>>(w, ns, F, shift, X, R);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rns_cheb2(const WaveDev& w, const long long* F, double* T2, int max_ld, cudaStream_t st) {
+  k_rns_cheb2<<<tile_grid(max_ld, w.nsub), 256, 0, st>>>(w, F, T2);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rns_cheb(const WaveDev& w, const RnsCheb& c, int max_ld, cudaStream_t st) {
+  if (c.odd) k_rns_cheb<true><<<tile_grid(max_ld, w.nsub), 256, 0, st>>>(w, c);
+  else k_rns_cheb<false><<<tile_grid(max_ld, w.nsub), 256, 0, st>>>(w, c);
   count_launch();
   return cudaGetLastError();
 }

@@ -69,4 +69,23 @@ cudaError_t launch_rns_square(const WaveDev& w, NsStateDev ns, const long long* 
 cudaError_t launch_rns_update(const WaveDev& w, NsStateDev ns, const long long* F, int shift, long long* X,
                               __nv_bfloat16* R, int max_ld, cudaStream_t st);
 
+// Chebyshev recurrences (fermi.cu).  All matrices have spectral norm 1 or less
+// and move as 2^-RNS_FRAC fixed point on their upper tiles.
+constexpr int RNS_COMB = 8;
+struct RnsCheb {
+  const long long* F;          // product, null: none
+  int twice;                   // 2 F instead of F
+  const long long* sub;        // subtracted (may be C), null: none
+  const long long* odd;        // RNS_COMB matrices, stride entries apart, null: none ...
+  int64_t stride;
+  long long coef[RNS_COMB];    // ... combined with these 2^-60 coefficients, and added
+  long long* C;                // the result (upper tiles), null: not stored
+  __nv_bfloat16* R;            // its residues (both triangles), null: none
+  double* out;                 // out_scale times the result, complete FP64 (may be C's memory), null: none
+  double out_scale;
+};
+cudaError_t launch_rns_cheb(const WaveDev& w, const RnsCheb& c, int max_ld, cudaStream_t st);
+// T2 = 2 X^2 - I, complete FP64, from X^2's sums.
+cudaError_t launch_rns_cheb2(const WaveDev& w, const long long* F, double* T2, int max_ld, cudaStream_t st);
+
 }  // namespace submat

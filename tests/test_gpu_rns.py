@@ -101,3 +101,42 @@ def test_exact_zero_eigenvalue(pkg):
     got, s = sign(pkg, m, 0.25, allow=True)
     assert s["not_converged"] == 1
     assert np.max(np.abs(got.reshape(3, 3) - np.diag([1.0, 0.5, 0.0]))) <= 1e-14
+
+
+def fermi(pkg, m, mu, kT, **kw):
+    import torch
+    K = torch.from_numpy(m.vals).cuda()
+    with pkg.Plan.from_bsr(m, prec="fp64", kT=kT, **kw) as plan:
+        D = plan.sign(K, mu, out=torch.zeros_like(K)).cpu().numpy()
+        return D, plan.stats()
+
+
+# tile edges, K beyond 1024, one Clenshaw block (kT 1) to many (kT 0.004: terms above 1)
+@pytest.mark.parametrize("n,kT", [(1, 0.1), (64, 0.01), (65, 1.0), (127, 0.05), (129, 0.02), (320, 0.05), (1025, 0.1)])
+def test_fermi_one_submatrix(pkg, n, kT):
+    m, a, st = one_submatrix(n, 70 + n)
+    w, q = np.linalg.eigh(a)
+    want = (q / (1.0 + np.exp(w / kT))) @ q.T
+    got, s = fermi(pkg, m, 0.0, kT, columns=(0, 1))
+    wide = np.concatenate([want[st[i]:st[i + 1], st[j]:st[j + 1]].ravel()
+                           for i in range(len(m.block_sizes)) for j in range(len(m.block_sizes))])
+    keep = got != 0
+    # truncation, and per product n * 3e-16 through 16 baby steps (T_16: 256) and the
+    # giant steps, whose errors grow with the derivative of f (at most 1 / (4 kT))
+    G = (s["poly_degree"] + 16) // 16
+    assert np.max(np.abs(got - wide)[keep]) <= 2e-13 + n * 3e-16 * (256 / (4 * kT) + G * G)
+    assert s["workspace_bytes"] >= 152 * ((n + 63) // 64 * 64) ** 2
+
+
+@pytest.mark.parametrize("form", [f for f in FORMS if f != "step cap"])
+@pytest.mark.parametrize("kT", [0.05, 0.4])
+def test_fermi_matches_simt_path(pkg, form, kT):
+    make, mu, kw = FORMS[form]
+    m = make()
+    got, s1 = fermi(pkg, m, mu, kT, **kw)
+    ld = (s1["n_max"] + 63) // 64 * 64
+    simt, s2 = fermi(pkg, m, mu, kT, workspace_cap_bytes=100 * ld * ld, **kw)
+    assert s2["workspace_bytes"] <= 100 * ld * ld < s1["workspace_bytes"]
+    G = (s1["poly_degree"] + 16) // 16
+    assert np.max(np.abs(got - simt)) <= 4e-13 + 2 * s1["n_max"] * 3e-16 * (256 / (4 * kT) + G * G)
+    assert abs(s1["dn_dmu"] - s2["dn_dmu"]) <= 1e-10 * m.n / kT
