@@ -34,9 +34,6 @@
 
 namespace submat {
 
-long long timeout_cycles_for(double seconds);
-int num_sms();
-
 // bytes of workspace per dense element (see MixedBufs)
 size_t mixed_bytes_per_elem() { return 8 + 8 + 4 + 8 + 8 + 4 + 4 + 4 + 4 * 4; }
 
@@ -1126,7 +1123,7 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
     SM_TRY(alloc(&ms->tol2, size_t(max_wave), "CG tolerances"));
     SM_TRY(alloc(&ms->submax, size_t(max_wave), "iterate maxima"));
   }
-  const long long tmo = timeout_cycles_for(2.0);
+  const long long tmo = kWaitCycles;
   const int nsm = num_sms();
   const double floor_thr = 1e-3;
   double* rr = ms->scal;
@@ -1808,7 +1805,7 @@ submat_status Plan::backward_wave_tc(size_t wi, const double* K, double mu, cons
     as->d_maps_b.push_back(d[1]);
   }
   const int nbk = int(wv.bucket_ld.size());
-  const long long tmo = timeout_cycles_for(2.0);
+  const long long tmo = kWaitCycles;
   const int nsm = num_sms();
   constexpr int bn = 256;
   const dim3 eg = elem_grid(wv);
