@@ -84,12 +84,11 @@ extern "C" submat_status submat_debug_tc_gemm(int count, int ld, int n, const vo
     for (int a = 0; a < T; ++a)
       for (int b = 0; b < TB; ++b)
         if (!sym || H * b + H - 1 >= a) items.push_back(make_int4(s, a, b, 0 | (s << 8)));
-  CUtensorMap maps[8];
+  CUtensorMap maps[4];
   std::memset(maps, 0, sizeof(maps));
   const void* srcs[4] = {A_hi, split ? A_lo : A_hi, B_hi, split ? B_lo : B_hi};
   for (int m = 0; m < 4; ++m)
-    if (make_bucket_map(&maps[m], srcs[m], ld, count) != 0 ||
-        make_bucket_map(&maps[4 + m], srcs[m], ld, count, 256) != 0) {
+    if (make_bucket_map(&maps[m], srcs[m], ld, count) != 0) {
       set_error("cuTensorMapEncodeTiled failed (map %d)", m);
       return SUBMAT_ERR_CUDA;
     }
@@ -108,7 +107,6 @@ extern "C" submat_status submat_debug_tc_gemm(int count, int ld, int n, const vo
   p.items = d_items;
   p.nitems = int(items.size());
   p.maps = d_maps;
-  p.maps_b = d_maps + 4;
   p.bn = bn;
   p.nbucket = 1;
   p.nmaps = 4;

@@ -30,6 +30,7 @@
 
 #include "pair.cuh"
 #include "plan.cuh"
+#include "slice_gemm.cuh"
 #include "tc_gemm.cuh"
 
 namespace submat {
@@ -265,8 +266,9 @@ __global__ void k_slice(WaveDev w, double* X, SlicePtrs out, int* __restrict__ r
 // 64-bit integers (Z + Z^T is even).  Written straight to the BF16 (hi, lo)
 // split that the next product reads.  32x32 tile pairs through shared memory;
 // block (8, 32): thread (x, y) owns columns 4x..4x+3 of row y.  S is on one
-// grid per submatrix, so every entry has the scale 2^(2 e - 48).
-__global__ void __launch_bounds__(256) k_hp_finalize_sym(WaveDev w, const long long* __restrict__ Z,
+// grid per submatrix, so every entry has the scale 2^(2 e - 48).  With whole
+// set, Z is S^2 itself, on its upper tiles.
+__global__ void __launch_bounds__(256) k_hp_finalize_sym(WaveDev w, const long long* __restrict__ Z, bool whole,
                                                          const int* __restrict__ ex,
                                                          const int64_t* __restrict__ voff,
                                                          __nv_bfloat16* hi, __nv_bfloat16* lo) {
@@ -287,16 +289,19 @@ __global__ void __launch_bounds__(256) k_hp_finalize_sym(WaveDev w, const long l
     const int64_t iba = base + int64_t(b * 32 + y) * ld + a * 32 + x4;
     const longlong2 z0 = *reinterpret_cast<const longlong2*>(Z + iab);
     const longlong2 z1 = *reinterpret_cast<const longlong2*>(Z + iab + 2);
-    const longlong2 z2 = *reinterpret_cast<const longlong2*>(Z + iba);
-    const longlong2 z3 = *reinterpret_cast<const longlong2*>(Z + iba + 2);
+    longlong2 z2, z3;
+    if (!whole) {
+      z2 = *reinterpret_cast<const longlong2*>(Z + iba);
+      z3 = *reinterpret_cast<const longlong2*>(Z + iba + 2);
+    }
     __syncthreads();
     ta_[y][x4] = z0.x; ta_[y][x4 + 1] = z0.y; ta_[y][x4 + 2] = z1.x; ta_[y][x4 + 3] = z1.y;
-    tb_[y][x4] = z2.x; tb_[y][x4 + 1] = z2.y; tb_[y][x4 + 2] = z3.x; tb_[y][x4 + 3] = z3.y;
+    if (!whole) { tb_[y][x4] = z2.x; tb_[y][x4 + 1] = z2.y; tb_[y][x4 + 2] = z3.x; tb_[y][x4 + 3] = z3.y; }
     __syncthreads();
     float v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const long long z = (ta_[y][x4 + k] + tb_[x4 + k][y]) >> 1;
+      const long long z = whole ? ta_[y][x4 + k] : (ta_[y][x4 + k] + tb_[x4 + k][y]) >> 1;
       double d = i64_to_f64_scaled(z, k2, true);
       if (a == b && y == x4 + k && a * 32 + y < n) d += 1.0;
       v[k] = d2f_trunc(d);
@@ -305,7 +310,7 @@ __global__ void __launch_bounds__(256) k_hp_finalize_sym(WaveDev w, const long l
     if (a != b) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const long long z = (tb_[y][x4 + k] + ta_[x4 + k][y]) >> 1;
+        const long long z = whole ? ta_[x4 + k][y] : (tb_[y][x4 + k] + ta_[x4 + k][y]) >> 1;
         v[k] = d2f_trunc(i64_to_f64_scaled(z, k2, true));
       }
       store_split4(make_float4(v[0], v[1], v[2], v[3]), hi, lo, iba);
@@ -958,7 +963,7 @@ dim3 pair_grid_stream(const Wave& wv) {
 
 struct MixedState {
   std::vector<CUtensorMap*> d_maps;  // per wave: [MS_COUNT][nbucket], 128-row boxes
-  std::vector<CUtensorMap*> d_maps_b;  // per wave: the same with 256-row boxes
+  std::vector<CUtensorMap*> d_maps32;  // per wave: the same with 32-column boxes (slice_gemm.cu)
   std::vector<int64_t*> d_voff;      // per wave: offset of each submatrix's row-scale vector
   int* rs_x = nullptr;               // row exponents of the first operand's slices
   int* rs_y = nullptr;               // row exponents of the second operand's slices
@@ -1073,38 +1078,24 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
     int64_t vec_max = 1;
     for (auto& wv : waves) {
       const int nbk = int(wv.bucket_ld.size());
-      std::vector<CUtensorMap> maps(size_t(MS_COUNT) * nbk);
       const void* bases[MS_COUNT] = {b.X[0][0], b.X[0][1], b.X[1][0], b.X[1][1], b.Y[0], b.Y[1],
                                      b.Ah[0],   b.Ah[1],   b.Hh[0],   b.Hh[1],   b.Z[0], b.Z[1]};
-      for (int m = 0; m < MS_COUNT; ++m)
-        for (int k = 0; k < nbk; ++k) {
-          const __nv_bfloat16* base = static_cast<const __nv_bfloat16*>(bases[m]) + wv.bucket_base[k];
-          if (make_bucket_map(&maps[size_t(m) * nbk + k], base, int(wv.bucket_ld[k]),
-                              wv.bucket_count[k]) != 0) {
-            set_error("cuTensorMapEncodeTiled failed");
-            return SUBMAT_ERR_CUDA;
+      for (int cols : {64, 32}) {
+        std::vector<CUtensorMap> maps(size_t(MS_COUNT) * nbk);
+        for (int m = 0; m < MS_COUNT; ++m)
+          for (int k = 0; k < nbk; ++k) {
+            const __nv_bfloat16* base = static_cast<const __nv_bfloat16*>(bases[m]) + wv.bucket_base[k];
+            if (make_bucket_map(&maps[size_t(m) * nbk + k], base, int(wv.bucket_ld[k]), wv.bucket_count[k], cols) !=
+                0) {
+              set_error("cuTensorMapEncodeTiled failed");
+              return SUBMAT_ERR_CUDA;
+            }
           }
-        }
-      CUtensorMap* d = nullptr;
-      SM_TRY(alloc(&d, maps.size(), "tensor maps"));
-      SM_CUDA(cudaMemcpyAsync(d, maps.data(), maps.size() * sizeof(CUtensorMap),
-                              cudaMemcpyHostToDevice, st));
-      ms->d_maps.push_back(d);
-      // the same sets with 256-row boxes for B operands of 128 x 256 tiles
-      for (int mset = 0; mset < MS_COUNT; ++mset)
-        for (int k = 0; k < nbk; ++k) {
-          const __nv_bfloat16* base = static_cast<const __nv_bfloat16*>(bases[mset]) + wv.bucket_base[k];
-          if (make_bucket_map(&maps[size_t(mset) * nbk + k], base, int(wv.bucket_ld[k]),
-                              wv.bucket_count[k], 256) != 0) {
-            set_error("cuTensorMapEncodeTiled failed");
-            return SUBMAT_ERR_CUDA;
-          }
-        }
-      CUtensorMap* db = nullptr;
-      SM_TRY(alloc(&db, maps.size(), "tensor maps"));
-      SM_CUDA(cudaMemcpyAsync(db, maps.data(), maps.size() * sizeof(CUtensorMap),
-                              cudaMemcpyHostToDevice, st));
-      ms->d_maps_b.push_back(db);
+        CUtensorMap* d = nullptr;
+        SM_TRY(alloc(&d, maps.size(), "tensor maps"));
+        SM_CUDA(cudaMemcpyAsync(d, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
+        (cols == 64 ? ms->d_maps : ms->d_maps32).push_back(d);
+      }
       std::vector<int64_t> vo(wv.count);
       int64_t acc = 0;
       for (int s = 0; s < wv.count; ++s) { vo[s] = acc; acc += wv.host_ld[s]; }
@@ -1157,7 +1148,6 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
       p.items = items;
       p.nitems = nitems;
       p.maps = ms->d_maps[wi];
-      p.maps_b = ms->d_maps_b[wi];
       p.bn = bn;
       p.nbucket = nbk;
       p.nmaps = MS_COUNT * nbk;
@@ -1325,7 +1315,9 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
     const dim3 slice_grid(unsigned(std::max<int64_t>(1, std::min<int64_t>(max_ld / 64, 256))), unsigned(wv.count));
     // C (+)= sign * X Y^T from the slices: level t = p + q weighs 2^(-6 t); each
     // launch sums at most per_acc products of one level in one exact accumulator
-    int hp_launch_products = 0;  // slice products issued (all residual products, this wave)
+    // slice products issued (all residual products, this wave): over 128 x 128
+    // tiles, and in one pass over all or the upper ones
+    int hp_launch_products = 0, hp_pass_full = 0, hp_pass_upper = 0;
     // out (int64) = sum over kept slice pairs (p, q), p + q <= 8, of
     // 2^(6 (8 - p - q)) X_p Y_q^T.  sym_pairs (X = Y, symmetric slices): only
     // p <= q, the p < q ones counted twice; the symmetric part of the sum is
@@ -1337,6 +1329,26 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
     // tiles per stage: fewer launches, so fewer int64 passes.
     auto hp_product = [&](const int* xs, int nx, const int* ys, int ny, bool sym_pairs,
                           double* out) -> submat_status {
+      if (slice_gemm_fits(nx, ny)) {  // one pass; X X^T from all pairs on its upper tiles
+        SliceGemmParams p{};
+        p.items = sym_pairs ? wv.sym128 : wv.full128;
+        p.nitems = sym_pairs ? wv.n_sym128 : wv.n_full128;
+        p.maps = ms->d_maps32[wi];
+        p.nbucket = nbk;
+        p.nx = nx; p.ny = ny;
+        for (int k = 0; k < nx; ++k) p.a_set[k] = xs[k];
+        for (int k = 0; k < ny; ++k) p.b_set[k] = ys[k];
+        p.off = wv.dev.off; p.ld = wv.dev.ld;
+        p.Z = reinterpret_cast<long long*>(out);
+        p.flags = d_flags;
+        p.timeout_cycles = tmo;
+        size_t tk;
+        SM_TRY(timer.start(KC_TC_HP, st, &tk));
+        SM_CUDA(launch_slice_gemm(p, nsm, st));
+        SM_TRY(timer.stop(tk, st));
+        (sym_pairs ? hp_pass_upper : hp_pass_full) += slice_gemm_products(nx, ny);
+        return SUBMAT_OK;
+      }
       // 128-wide tiles carry up to four accumulators (all of TMEM, single-
       // buffered, combined in 64-bit integers); 256-wide ones two
       const int want_w = opt.tile_n_hp == 256 ? 256 : 128;
@@ -1359,8 +1371,7 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
         p.items = FULL;
         p.nitems = NFULL;
         p.maps = ms->d_maps[wi];
-        p.maps_b = ms->d_maps_b[wi];
-        p.bn = bn;
+          p.bn = bn;
         p.nbucket = nbk;
         p.nmaps = MS_COUNT * nbk;
         p.na = na; p.nb = nb;
@@ -1437,7 +1448,8 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
         SM_TRY(hp_product(S_SETS, s_keep, S_SETS, s_keep, true, b.T));
         // (I - S^2) straight to its split in Y
         k_hp_finalize_sym<<<pair_grid_stream(wv), dim3(8, 32), 0, st>>>(
-            wv.dev, reinterpret_cast<const long long*>(b.T), ms->rs_x, ms->d_voff[wi], b.Y[0], b.Y[1]);
+            wv.dev, reinterpret_cast<const long long*>(b.T), slice_gemm_fits(s_keep, s_keep), ms->rs_x, ms->d_voff[wi],
+            b.Y[0], b.Y[1]);
         SM_KCHECK();
       } else {
         // S's BF16 split for the correction products (in the first round X0
@@ -1675,7 +1687,8 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
       stats.kernel_exec[KC_TC_NS] += (third ? 3.0 : 2.0) * lp_iters[s] * 3.0 * sym_tiles_ns * tile_ns;
       const double symt = t128 * (t128 + 1) / 2, fullt = t128 * t128;
       stats.kernel_exec[KC_TC_REF] += rounds * 3.0 * (2.0 * symt + fullt) * tile128 + cgc[s] * 3.0 * fullt * tile128;
-      if (hp_sliced) stats.kernel_exec[KC_TC_HP] += double(hp_launch_products) * fullt * tile128;
+      if (hp_sliced)
+        stats.kernel_exec[KC_TC_HP] += ((hp_launch_products + hp_pass_full) * fullt + hp_pass_upper * symt) * tile128;
     }
     stats.refine_fallback = fallback_total;
   }
@@ -1705,7 +1718,7 @@ enum AdjSet {
 };
 
 struct AdjState {
-  std::vector<CUtensorMap*> d_maps, d_maps_b;  // per adjoint wave: [AS_COUNT][nbucket]
+  std::vector<CUtensorMap*> d_maps;  // per adjoint wave: [AS_COUNT][nbucket]
 };
 
 // dst = src^T for a BF16 (hi, lo) pair (src and dst distinct): 32x32 tile
@@ -1782,27 +1795,23 @@ submat_status Plan::backward_wave_tc(size_t wi, const double* K, double mu, cons
     as = new AdjState();
     adj_tc = as;
   }
-  // tensor maps of every adjoint wave (128-row boxes; 256-row boxes for the
-  // B operands of 128 x 256 tiles), built once
+  // tensor maps of every adjoint wave, built once
   while (as->d_maps.size() < bwaves.size()) {
     const Wave& mw = bwaves[as->d_maps.size()];
     const int nb2 = int(mw.bucket_ld.size());
-    CUtensorMap* d[2] = {nullptr, nullptr};
-    for (int v = 0; v < 2; ++v) {
-      std::vector<CUtensorMap> maps(size_t(AS_COUNT) * nb2);
-      for (int m = 0; m < AS_COUNT; ++m)
-        for (int k = 0; k < nb2; ++k)
-          if (make_bucket_map(&maps[size_t(m) * nb2 + k], P[m] + mw.bucket_base[k], int(mw.bucket_ld[k]),
-                              mw.bucket_count[k], v ? 256 : 128) != 0) {
-            set_error("cuTensorMapEncodeTiled failed");
-            return SUBMAT_ERR_CUDA;
-          }
-      SM_TRY(alloc(&d[v], maps.size(), "tensor maps"));
-      SM_CUDA(cudaMemcpyAsync(d[v], maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
-      SM_CUDA(cudaStreamSynchronize(st));  // the host array goes out of scope
-    }
-    as->d_maps.push_back(d[0]);
-    as->d_maps_b.push_back(d[1]);
+    CUtensorMap* d = nullptr;
+    std::vector<CUtensorMap> maps(size_t(AS_COUNT) * nb2);
+    for (int m = 0; m < AS_COUNT; ++m)
+      for (int k = 0; k < nb2; ++k)
+        if (make_bucket_map(&maps[size_t(m) * nb2 + k], P[m] + mw.bucket_base[k], int(mw.bucket_ld[k]),
+                            mw.bucket_count[k]) != 0) {
+          set_error("cuTensorMapEncodeTiled failed");
+          return SUBMAT_ERR_CUDA;
+        }
+    SM_TRY(alloc(&d, maps.size(), "tensor maps"));
+    SM_CUDA(cudaMemcpyAsync(d, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
+    SM_CUDA(cudaStreamSynchronize(st));  // the host array goes out of scope
+    as->d_maps.push_back(d);
   }
   const int nbk = int(wv.bucket_ld.size());
   const long long tmo = kWaitCycles;
@@ -1818,7 +1827,6 @@ submat_status Plan::backward_wave_tc(size_t wi, const double* K, double mu, cons
     p.items = items;
     p.nitems = nitems;
     p.maps = as->d_maps[wi];
-    p.maps_b = as->d_maps_b[wi];
     p.bn = bn;
     p.nbucket = nbk;
     p.nmaps = AS_COUNT * nbk;

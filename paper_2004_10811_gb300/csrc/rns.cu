@@ -99,27 +99,6 @@ constexpr int SMEM = 1024 + STAGES * 2 * TILE + (2 * STAGES + 2 * NBUF + 1) * 8 
 // D F32, A and B BF16, both K-major, M = N = 128
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(TM >> 3) << 17) | (uint32_t(TM >> 4) << 24);
 
-// sixteen consecutive TMEM columns of this thread's lane; valid after tmem_wait16
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
-      "%12, %13, %14, %15}, [%16];"
-      : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
-        "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
-      : "r"(taddr));
-}
-
-// waits for this thread's TMEM loads; the values pass through, so that nothing
-// reads them earlier
-__device__ __forceinline__ void tmem_wait16(float* r) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(r[0]), "+f"(r[1]), "+f"(r[2]), "+f"(r[3]), "+f"(r[4]), "+f"(r[5]), "+f"(r[6]), "+f"(r[7]),
-                 "+f"(r[8]), "+f"(r[9]), "+f"(r[10]), "+f"(r[11]), "+f"(r[12]), "+f"(r[13]), "+f"(r[14]),
-                 "+f"(r[15])
-               :
-               : "memory");
-}
-
 // f += r w modulo 2^64: one wide multiply-add and one for the upper half
 __device__ __forceinline__ void add_weighted(unsigned long long& f, uint32_t r, uint32_t wlo, uint32_t whi) {
   asm("{\n\t.reg .u32 lo, hi;\n\t.reg .u64 t;\n\t"

@@ -11,9 +11,9 @@
 // the three-term split hi*hi + hi*lo + lo*hi that carries about 16 bits
 // through the tensor cores.
 //
-// Roles (192 threads): warp 0 issues TMA loads, warp 1 owns TMEM and one of
-// its lanes issues the MMAs, warps 2-5 drain the accumulator (one TMEM lane
-// quarter each) and write the tile -- and, for symmetric outputs, its mirror
+// Roles (192 or 320 threads): warp 0 issues TMA loads, warp 1 owns TMEM and one of
+// its lanes issues the MMAs, warps 2-5 (or 2-9) drain the accumulator (one TMEM
+// lane quarter each, or half of one) and write the tile -- and, for symmetric outputs, its mirror
 // through a shared-memory transpose.  Every mbarrier wait is bounded; on
 // timeout the kernel raises FLAG_TIMEOUT, drains its own copies and MMAs,
 // frees TMEM and returns.
@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "tc_gemm.cuh"
 #include "tcgen05.cuh"
@@ -40,11 +41,21 @@ constexpr int STG_PITCH = 33;            // staged row pitch (32-bit words)
 constexpr int I64_SEG = 16, I64_PITCH = 144;
 constexpr int STG_BYTES = (BM * I64_PITCH > BM * STG_PITCH * 4) ? BM * I64_PITCH : BM * STG_PITCH * 4;
 
-// instruction descriptor: D F32, A and B BF16, both K-major, M = 128, N = BN
+// instruction descriptor: D F32, A and B BF16, both K-major, M = 128, N = cols
 // (FP16 operands clear the two format fields, bits 7-9 and 10-12)
+__device__ __forceinline__ constexpr uint32_t idesc(int cols) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(cols >> 3) << 17) | (uint32_t(BM >> 4) << 24);
+}
+
+// Columns of a tile that its MMAs form: those inside the matrix (ld is a
+// multiple of 64), and of a 256-wide tile of a symmetric result whose left half
+// lies below the diagonal the right half only.
+struct TileCols {
+  int lo, hi;
+};
 template <int BN>
-__device__ __forceinline__ constexpr uint32_t idesc() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN >> 3) << 17) | (uint32_t(BM >> 4) << 24);
+__device__ __forceinline__ TileCols tile_cols(const int4& item, int ld, int sym) {
+  return TileCols{BN == 256 && sym && item.z * 2 < item.y ? 128 : 0, min(BN, ld - item.z * BN)};
 }
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -177,12 +188,29 @@ __device__ __forceinline__ void load_c0(const TcGemmParams& p, int64_t idx, floa
   }
 }
 
-// LEAN: the launch has one accumulator, a BF16-pair or FP32 output, no
-// mirror and double-buffered TMEM (the host checks), and the epilogue drains
-// it 32 columns at a time; the general epilogue is not compiled in.
-template <int BN, bool LEAN, bool F16>
-__global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGemmParams p) {
+// The epilogue a launch compiles in (the host checks what each needs):
+// EPI_GENERAL anything, the tile's 128 columns live in registers; EPI_FLOAT one
+// accumulator, a 16-bit pair or FP32 output, no mirror, double-buffered TMEM;
+// EPI_INT integer sums of slice products.  The last two drain 32 columns at a
+// time.
+// EPI_FLOAT has eight epilogue warps, two for each TMEM lane quarter, which take
+// the chunks in turn: with four, converting and storing a tile of few k-blocks
+// took longer than its MMAs (1000 FP16 products of 192 dims: 129 -> 111 us, and
+// 83 us at a width of 256).
+enum Epilogue { EPI_GENERAL, EPI_FLOAT, EPI_INT };
+__host__ __device__ constexpr int epi_warps(int mode) { return mode == EPI_FLOAT ? 8 : 4; }
+
+// hi + lo += x, both FP32, with the rounding error kept
+__device__ __forceinline__ void add_pair(float x, float& hi, float& lo) {
+  const float s = hi + x, b = s - hi;
+  lo += (hi - (s - b)) + (x - b);
+  hi = s;
+}
+
+template <int BN, int MODE, bool F16>
+__global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const __grid_constant__ TcGemmParams p) {
   constexpr int TILE_B = BN * BK * 2;  // one BN x 64 BF16 operand tile (B side)
+  constexpr bool LEAN = MODE != EPI_GENERAL;
   constexpr int HALVES = BN / 128;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -208,7 +236,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGe
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], BM);
+      mbar_init(&tempty[i], 32 * epi_warps(MODE));
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -241,19 +269,23 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGe
       const int4 item = p.items[it];
       if (p.state && p.state[item.x] == p.skip_state) continue;
       const int bucket = item.w & 0xFF, slot = item.w >> 8;
-      const int nk = p.ld[item.x] / BK;
-      const CUtensorMap* mapsa = p.maps + bucket;
-      const CUtensorMap* mapsb = (BN == 128 ? p.maps : p.maps_b) + bucket;
+      const int ld = p.ld[item.x], nk = ld / BK;
+      const CUtensorMap* maps = p.maps + bucket;
+      // 128-row boxes of the B tile that hold wanted columns
+      const TileCols tc = tile_cols<BN>(item, ld, p.sym);
+      const int box0 = tc.lo / 128, box1 = (tc.hi + 127) / 128;
+      const uint32_t bytes = uint32_t(p.na + p.nb * (box1 - box0)) * TILE_BYTES;
       for (int kb = 0; kb < nk; ++kb) {
         if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, limit)) { ok = false; break; }
         uint8_t* st = tiles + size_t(stage) * stage_bytes;
-        mbar_expect_tx(&full[stage], uint32_t(stage_bytes));
+        mbar_expect_tx(&full[stage], bytes);
         for (int a = 0; a < p.na; ++a)
-          tma_load_3d(st + a * TILE_BYTES, mapsa + p.a_set[a] * p.nbucket, &full[stage], kb * BK,
+          tma_load_3d(st + a * TILE_BYTES, maps + p.a_set[a] * p.nbucket, &full[stage], kb * BK,
                       item.y * BM, slot);
         for (int b = 0; b < p.nb; ++b)
-          tma_load_3d(st + p.na * TILE_BYTES + b * TILE_B, mapsb + p.b_set[b] * p.nbucket,
-                      &full[stage], kb * BK, item.z * BN, slot);
+          for (int x = box0; x < box1; ++x)
+            tma_load_3d(st + p.na * TILE_BYTES + b * TILE_B + x * TILE_BYTES, maps + p.b_set[b] * p.nbucket,
+                        &full[stage], kb * BK, item.z * BN + x * 128, slot);
         issued |= 1u << stage;
         issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
         if (++stage == p.nstage) { stage = 0; phase ^= 1u; }
@@ -279,20 +311,16 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGe
     for (int it = blockIdx.x; it < p.nitems && ok; it += gridDim.x) {
       const int4 item = p.items[it];
       if (p.state && p.state[item.x] == p.skip_state) continue;
-      const int nk = p.ld[item.x] / BK;
+      const int ld = p.ld[item.x], nk = ld / BK;
       const int ab = nbuf == 2 ? (tcount & 1) : 0;
       const uint32_t tph = nbuf == 2 ? (uint32_t(tcount >> 1) & 1u) : (uint32_t(tcount) & 1u);
       if (!mbar_wait(&tempty[ab], tph ^ 1u, abort_flag, limit)) { ok = false; break; }
       tc_fence_after();
       const uint32_t dbase = tmem_base + uint32_t(ab * p.nacc * BN);
-      // symmetric output, 256-wide tile whose left 128 columns lie below the
-      // diagonal (odd row block): only the right half is wanted, so the MMAs
-      // run at N = 128 on B rows 128..255 into accumulator columns 128..255
-      const bool half = BN == 256 && p.sym && item.z * 2 < item.y;
+      const TileCols tc = tile_cols<BN>(item, ld, p.sym);
       // operand format: BF16 (A and B fields 1) or FP16 (both 0)
-      const uint32_t id = (half ? idesc<128>() : idesc<BN>()) & (F16 ? ~((7u << 7) | (7u << 10)) : ~0u);
-      const uint32_t boff = half ? uint32_t(128 * BK * 2) : 0u;
-      const uint32_t doff = half ? 128u : 0u;
+      const uint32_t id = idesc(tc.hi - tc.lo) & (F16 ? ~((7u << 7) | (7u << 10)) : ~0u);
+      const uint32_t boff = uint32_t(tc.lo * BK * 2), doff = uint32_t(tc.lo);
       for (int kb = 0; kb < nk; ++kb) {
         if (!mbar_wait(&full[stage], phase, abort_flag, limit)) { ok = false; break; }
         tc_fence_after();
@@ -333,17 +361,26 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGe
       if (p.state && p.state[s] == p.skip_state) continue;
       const int ab = nbuf == 2 ? (tcount & 1) : 0;
       const uint32_t tph = nbuf == 2 ? (uint32_t(tcount >> 1) & 1u) : (uint32_t(tcount) & 1u);
-      // one bounded wait, result shared, so the four warps leave together
-      if (threadIdx.x == 64) {
-        const bool got = mbar_wait(&tfull[ab], tph, abort_flag, limit);
-        if (!got) {
-          atomicOr(p.flags, FLAG_TIMEOUT);
+      if constexpr (MODE == EPI_FLOAT) {
+        // no shared memory to agree on: every warp waits by itself
+        if (!__all_sync(0xffffffffu, mbar_wait(&tfull[ab], tph, abort_flag, limit))) {
+          if (lane == 0) atomicOr(p.flags, FLAG_TIMEOUT);
           *abort_flag = 1;
+          break;
         }
-        *epi_ok = got ? 1 : 0;
+      } else {
+        // one bounded wait, result shared, so the four warps leave together
+        if (threadIdx.x == 64) {
+          const bool got = mbar_wait(&tfull[ab], tph, abort_flag, limit);
+          if (!got) {
+            atomicOr(p.flags, FLAG_TIMEOUT);
+            *abort_flag = 1;
+          }
+          *epi_ok = got ? 1 : 0;
+        }
+        epi_bar();
+        if (!*epi_ok) break;
       }
-      epi_bar();
-      if (!*epi_ok) break;
       tc_fence_after();
       ++tcount;
       const int ld = p.ld[s];
@@ -352,12 +389,11 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGe
       const int rg = item.y * BM + r;
       double part = 0.0;
       const uint32_t tbase = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(ab * p.nacc * BN);
-      // Lean path for the common launches (one accumulator, BF16-pair or FP32
-      // output, no mirror, double-buffered TMEM): 32 columns at a time, so
-      // only one chunk is live in registers, and the diagonal handled only
-      // on diagonal sub-tiles.  TMEM is released after its last read.
+      // 32 columns at a time, so only one chunk is live in registers, and the
+      // diagonal handled only on diagonal sub-tiles.  TMEM is released after its
+      // last read.
       if constexpr (LEAN) {
-        if (p.out_i64) {
+        if constexpr (MODE == EPI_INT) {
           // exact integer sums of slice products (full tiles): per 32-column
           // chunk the sum over the accumulators of acc_k * 2^shift_k in 64-bit
           // integers (|acc_k| < 2^24, shift_k <= 36, at most four terms),
@@ -403,34 +439,31 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGe
               asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
           }
-        } else
-        for (int h = 0; h < HALVES; ++h) {
-          const int sub_tj = item.z * HALVES + h;
-          const bool last_h = h == HALVES - 1;
-          if (p.sym && sub_tj < item.y) {  // below the diagonal: not written
-            if (last_h) {
-              tc_fence_before();
-              if (!p.test_skip_arrive) mbar_arrive(&tempty[ab]);
-            }
-            continue;
-          }
-          const bool dtile = item.y == sub_tj;  // the diagonal crosses this sub-tile
-          const bool diag_sym = p.sym && dtile;
-          const double res_weight = (p.sym && !diag_sym) ? 2.0 : 1.0;
-          const uint32_t tb = tbase + uint32_t(h * 128);
+        } else {
+          const int side = (warp - 2) >> 2;  // chunks side, side + 2, ...
+          const bool has_c0 = (p.c0_f32 || p.c0_hi) && p.beta != 0.0f && !p.dot_c0;
+          float ph = 0.0f, pl = 0.0f;  // the tile's sum for res2 or dot_c0
 #pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
+          for (int hc = side; hc < 4 * HALVES; hc += 2) {
+            const int h = hc >> 2, c = hc & 3;
+            const int sub_tj = item.z * HALVES + h;
+            // below the diagonal or beyond the matrix: not formed, not written
+            const bool skip = (p.sym && sub_tj < item.y) || sub_tj * 128 + c * 32 >= ld;
             float a[32];
-            tmem_ld32(tb + uint32_t(c * 32), a);
-            tmem_wait_ld();
-            if (last_h && c == 3) {
+            if (!skip) {
+              tmem_ld32(tbase + uint32_t(hc * 32), a);
+              tmem_wait_ld();
+            }
+            if (hc >= 4 * HALVES - 2) {
               tc_fence_before();
               if (!p.test_skip_arrive) mbar_arrive(&tempty[ab]);
             }
+            if (skip) continue;
+            const bool dtile = item.y == sub_tj;  // the diagonal crosses this sub-tile
+            const bool diag_sym = p.sym && dtile;
             const int cg0 = sub_tj * 128 + c * 32;
-            if (rg >= ld || cg0 >= ld) continue;
+            if (rg >= ld) continue;
             const int64_t idx = base + int64_t(rg) * ld + cg0;
-            const bool has_c0 = (p.c0_f32 || p.c0_hi) && p.beta != 0.0f && !p.dot_c0;
             float c0[32];
             if (has_c0 || p.dot_c0) load_c0<F16>(p, idx, c0);
             float o[32];
@@ -457,10 +490,24 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGe
                 if (p.dot_c0) pd = fmaf(v, c0[q], pd);
               }
             }
-            if (p.res2) part += res_weight * double(pr);
-            if (p.dot_c0) part += 2.0 * double(pd);
+            if (p.res2) add_pair(p.sym && !diag_sym ? 2.0f * pr : pr, ph, pl);
+            if (p.dot_c0) add_pair(2.0f * pd, ph, pl);
             if (diag_sym) store_range<F16>(p, idx, o, r - c * 32, 32);
             else store_row<F16>(p, idx, o);
+          }
+          // FP64 instructions hold their pipe for 64 clocks: sums stay in FP32
+          // pairs up to one conversion per warp
+          if (p.res2 || p.dot_c0) {
+#pragma unroll
+            for (int o2 = 16; o2 > 0; o2 >>= 1) {
+              const float xh = __shfl_xor_sync(0xffffffffu, ph, o2), xl = __shfl_xor_sync(0xffffffffu, pl, o2);
+              add_pair(xh, ph, pl);
+              pl += xl;
+            }
+            if (lane == 0) {
+              const double t = double(ph) + double(pl);
+              if (t != 0.0) atomicAdd(p.res2 ? &p.res2[s] : &p.dot_c0[s], t);
+            }
           }
         }
       } else {
@@ -605,7 +652,7 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm(const __grid_constant__ TcGe
       }
       }  // halves
       }  // general epilogue
-      if (p.res2 || p.dot_c0) {
+      if (!LEAN && (p.res2 || p.dot_c0)) {
 #pragma unroll
         for (int o2 = 16; o2 > 0; o2 >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o2);
         if (lane == 0 && part != 0.0) atomicAdd(p.res2 ? &p.res2[s] : &p.dot_c0[s], part);
@@ -639,7 +686,7 @@ int tc_pick_stages(int na, int nb, int bn) {
 cudaError_t launch_tc_gemm(const TcGemmParams& p, int grid, cudaStream_t st) {
   if (p.nitems <= 0) return cudaSuccess;
   const int bn = p.bn == 256 ? 256 : 128;
-  if (bn == 256 && (p.tmem_cols != 512 || !p.maps_b || !(p.nacc == 1 || (p.nacc == 2 && p.out_i64))))
+  if (bn == 256 && (p.tmem_cols != 512 || !(p.nacc == 1 || (p.nacc == 2 && p.out_i64))))
     return cudaErrorInvalidValue;
   if (p.nacc * bn > p.tmem_cols) return cudaErrorInvalidValue;
   if (p.out_i64 && p.sym) return cudaErrorInvalidValue;  // integer outputs: full tiles only
@@ -659,21 +706,24 @@ cudaError_t launch_tc_gemm(const TcGemmParams& p, int grid, cudaStream_t st) {
   const bool lean = (p.out_i64 ? lean_i64
                                 : p.tmem_cols >= 2 * bn && p.nacc == 1 && !(p.sym && !p.upper_only) &&
                                       (p.out_f32 || p.out_hi));
-  auto run = [&](auto kern) -> cudaError_t {
+  auto run = [&](auto kern, int mode) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, 192, smem, st>>>(p);
+    kern<<<grid, 64 + 32 * epi_warps(mode), smem, st>>>(p);
     return cudaSuccess;
   };
   // FP16 operands: lean launches only (the Newton-Schulz products)
   if (p.f16 && !lean) return cudaErrorInvalidValue;
+  if (p.f16 && p.out_i64) return cudaErrorInvalidValue;
   cudaError_t e;
-  if (bn == 256)
-    e = p.f16 ? run(k_tc_gemm<256, true, true>)
-              : (lean ? run(k_tc_gemm<256, true, false>) : run(k_tc_gemm<256, false, false>));
-  else
-    e = p.f16 ? run(k_tc_gemm<128, true, true>)
-              : (lean ? run(k_tc_gemm<128, true, false>) : run(k_tc_gemm<128, false, false>));
+  auto pick = [&](auto width) -> cudaError_t {
+    constexpr int W = decltype(width)::value;
+    if (p.f16) return run(k_tc_gemm<W, EPI_FLOAT, true>, EPI_FLOAT);
+    if (!lean) return run(k_tc_gemm<W, EPI_GENERAL, false>, EPI_GENERAL);
+    if (p.out_i64) return run(k_tc_gemm<W, EPI_INT, false>, EPI_INT);
+    return run(k_tc_gemm<W, EPI_FLOAT, false>, EPI_FLOAT);
+  };
+  e = bn == 256 ? pick(std::integral_constant<int, 256>()) : pick(std::integral_constant<int, 128>());
   if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
@@ -701,15 +751,16 @@ static PFN_encodeTiled get_encoder() {
   return fn;
 }
 
-int make_bucket_map(CUtensorMap* out, const void* base, int ld, int count, int box_rows) {
+int make_bucket_map(CUtensorMap* out, const void* base, int ld, int count, int box_k) {
   PFN_encodeTiled enc = get_encoder();
   if (!enc) return -1;
   const cuuint64_t dims[3] = {cuuint64_t(ld), cuuint64_t(ld), cuuint64_t(count)};
   const cuuint64_t strides[2] = {cuuint64_t(ld) * 2, cuuint64_t(ld) * ld * 2};
-  const cuuint32_t box[3] = {BK, cuuint32_t(box_rows), 1};
+  const cuuint32_t box[3] = {cuuint32_t(box_k), BM, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
-                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   box_k == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : int(r);
 }

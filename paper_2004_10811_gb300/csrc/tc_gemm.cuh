@@ -17,8 +17,7 @@ constexpr int TC_MAX_PROD = 16;
 struct TcGemmParams {
   const int4* items;        // (s, ti, tj, bucket | slot << 8), 128 x 128 tiles
   int nitems;
-  const CUtensorMap* maps;  // device array [set][bucket], 128-row boxes (A operands; B when bn = 128)
-  const CUtensorMap* maps_b;  // same sets with 256-row boxes (B operands when bn = 256)
+  const CUtensorMap* maps;  // device array [set][bucket], 128-row boxes
   int bn;                   // output tile width: 128 or 256 (then tmem_cols = 512: nacc = 1 double-
                             // buffered, or nacc = 2 integer accumulators single-buffered)
   int nbucket, nmaps;
@@ -71,7 +70,8 @@ struct TcGemmParams {
 int tc_smem_bytes(int na, int nb, int nstage, int bn = 128);
 int tc_pick_stages(int na, int nb, int bn = 128);
 cudaError_t launch_tc_gemm(const TcGemmParams& p, int grid, cudaStream_t st);
-// 3D map over a bucket [count][ld][ld] of BF16, box 64 x box_rows x 1, 128B swizzle.
-int make_bucket_map(CUtensorMap* out, const void* base, int ld, int count, int box_rows = 128);
+// 3D map over a bucket [count][ld][ld] of BF16, box box_k x 128 x 1, swizzled over
+// the box's row: 128 bytes (box_k 64) or 64 (32).
+int make_bucket_map(CUtensorMap* out, const void* base, int ld, int count, int box_k = 64);
 
 }  // namespace submat
