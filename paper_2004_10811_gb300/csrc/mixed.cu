@@ -502,74 +502,8 @@ __device__ __forceinline__ double block_sum(float v, double* red) {
   return t;
 }
 
-// Complete a symmetric BF16 (hi, lo) pair from its upper triangle: entry
-// (r, c), r > c, takes (c, r).  32x32 tile pairs, two per iteration so that
-// twice the loads are in flight; block (8, 32).
-__global__ void __launch_bounds__(256) k_mirror_split(WaveDev w, __nv_bfloat16* hi, __nv_bfloat16* lo,
-                                                      const int* __restrict__ state, int skip_state) {
-  __shared__ uint32_t th[2][32][33], tl[2][32][33];  // BF16 bits of the upper tiles
-  const int s = blockIdx.y;
-  if (state && state[s] == skip_state) return;
-  const int ld = w.ld[s];
-  const int64_t base = w.off[s];
-  const int T = ld / 32;
-  const int npair = T * (T + 1) / 2;
-  const int x4 = threadIdx.x * 4, y = threadIdx.y;
-  const unsigned short* h16 = reinterpret_cast<const unsigned short*>(hi);
-  const unsigned short* l16 = reinterpret_cast<const unsigned short*>(lo);
-  for (int p0 = blockIdx.x; p0 < npair; p0 += 2 * gridDim.x) {
-    int ta[2], tb[2];
-    uint2 hv[2], lv[2];
-    const int np = p0 + int(gridDim.x) < npair ? 2 : 1;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (q < np) {
-        int a = 0, rem = p0 + q * int(gridDim.x);
-        while (rem >= T - a) { rem -= T - a; ++a; }
-        ta[q] = a; tb[q] = a + rem;  // upper tile (a, b), a <= b; lower tile (b, a)
-        const int64_t iab = base + int64_t(a * 32 + y) * ld + tb[q] * 32 + x4;
-        hv[q] = *reinterpret_cast<const uint2*>(h16 + iab);
-        lv[q] = *reinterpret_cast<const uint2*>(l16 + iab);
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (q < np) {
-        th[q][y][x4] = hv[q].x & 0xFFFFu; th[q][y][x4 + 1] = hv[q].x >> 16;
-        th[q][y][x4 + 2] = hv[q].y & 0xFFFFu; th[q][y][x4 + 3] = hv[q].y >> 16;
-        tl[q][y][x4] = lv[q].x & 0xFFFFu; tl[q][y][x4 + 1] = lv[q].x >> 16;
-        tl[q][y][x4 + 2] = lv[q].y & 0xFFFFu; tl[q][y][x4 + 3] = lv[q].y >> 16;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (q >= np) continue;
-      const int a = ta[q], b = tb[q];
-      // lower tile (b, a), row y, columns x4..x4+3 = upper (a, b) column y, rows x4..x4+3
-      const int64_t iba = base + int64_t(b * 32 + y) * ld + a * 32 + x4;
-      if (a != b) {
-        *reinterpret_cast<uint2*>(hi + iba) = make_uint2(th[q][x4][y] | (th[q][x4 + 1][y] << 16),
-                                                         th[q][x4 + 2][y] | (th[q][x4 + 3][y] << 16));
-        *reinterpret_cast<uint2*>(lo + iba) = make_uint2(tl[q][x4][y] | (tl[q][x4 + 1][y] << 16),
-                                                         tl[q][x4 + 2][y] | (tl[q][x4 + 3][y] << 16));
-      } else {
-        // diagonal tile: only its strict lower triangle (row y > column x4 + k)
-        unsigned short* hd = reinterpret_cast<unsigned short*>(hi) + iba;
-        unsigned short* ld16 = reinterpret_cast<unsigned short*>(lo) + iba;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (y > x4 + k) {
-            hd[k] = static_cast<unsigned short>(th[q][x4 + k][y]);
-            ld16[k] = static_cast<unsigned short>(tl[q][x4 + k][y]);
-          }
-      }
-    }
-  }
-}
-
-// The same for a symmetric FP32 matrix.
+// Complete a symmetric FP32 matrix from its upper triangle: entry (r, c), r > c,
+// takes (c, r).  32x32 tile pairs, block (8, 32).
 __global__ void __launch_bounds__(256) k_mirror_f32(WaveDev w, float* C) {
   __shared__ float t[32][33];
   const int s = blockIdx.y;
@@ -1223,11 +1157,8 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
       g1.out_hi = b.Y[0]; g1.out_lo = b.Y[1];
       g1.res2 = ns.res2;
       g1.state = ns.state; g1.skip_state = ST_DONE;
-      g1.upper_only = 1;
       g1.f16 = 1;
       SM_CUDA(launch(g1));
-      k_mirror_split<<<pair_grid_stream(wv), dim3(8, 32), 0, st>>>(wv.dev, b.Y[0], b.Y[1], ns.state, ST_DONE);
-      SM_KCHECK();
       if (k == 0 && opt.beta_mode == 0) {  // the power estimate's scale, proven from X_0^2 or reduced
         const CertSquare sq{3, b.Y[0], b.Y[1], g1.alpha, g1.diag};
         const CertLinear lin{1, {b.X[0][0], nullptr, nullptr}, {b.X[0][1], nullptr, nullptr}};
@@ -1240,23 +1171,16 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
         gw.diag = 5.0f / 6.0f;
         gw.out_hi = b.Hh[0]; gw.out_lo = b.Hh[1];
         gw.state = ns.state; gw.skip_state = ST_DONE;
-        gw.upper_only = 1;
         gw.f16 = 1;
         SM_CUDA(launch(gw));
-        k_mirror_split<<<pair_grid_stream(wv), dim3(8, 32), 0, st>>>(wv.dev, b.Hh[0], b.Hh[1], ns.state, ST_DONE);
-        SM_KCHECK();
         z_hi = MS_HH;
         z_lo = MS_HL;
       }
       TcGemmParams g2 = tc(SYM, NSYM, cur ? MS_XH1 : MS_XH0, cur ? MS_XL1 : MS_XL0, z_hi, z_lo, 1, 1.0f, 0.0f);
       g2.out_hi = b.X[cur ^ 1][0]; g2.out_lo = b.X[cur ^ 1][1];
       g2.state = ns.state; g2.skip_state = ST_DONE;
-      g2.upper_only = 1;
       g2.f16 = 1;
       SM_CUDA(launch(g2));
-      k_mirror_split<<<pair_grid_stream(wv), dim3(8, 32), 0, st>>>(wv.dev, b.X[cur ^ 1][0], b.X[cur ^ 1][1], ns.state,
-                                                           ST_DONE);
-      SM_KCHECK();
       SM_CUDA(cudaMemsetAsync(d_active, 0, sizeof(int), st));
       SM_CUDA(launch_ns_post(wv.dev, ns, cur ^ 1, d_active, st));
       SM_CUDA(cudaMemcpyAsync(h_pinned, d_active, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1399,8 +1323,6 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
         p.flags = d_flags;
         p.timeout_cycles = tmo;
         p.out_i64 = reinterpret_cast<long long*>(out);
-        p.i64_shift = L.ng == 2 ? gs[1]->shift : gs[0]->shift;
-        p.i64_dshift = L.ng == 2 ? gs[0]->shift - gs[1]->shift : 0;
         p.i64_accumulate = first ? 0 : 1;
         const int saved = tc_class;
         tc_class = KC_TC_HP;
@@ -1469,10 +1391,7 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
       // F_c = -1/2 S (I - S^2)
       TcGemmParams g = tc(SYM, NSYM, s_hi, s_lo, MS_YH, MS_YL, 1, -0.5f, 0.0f);
       g.out_f32 = b.Fc;
-      g.upper_only = 1;
       SM_CUDA(launch(g));
-      k_mirror_f32<<<pair_grid_stream(wv), dim3(8, 32), 0, st>>>(wv.dev, b.Fc);
-      SM_KCHECK();
       // W = F_c a, before S a so that a's split and Y are free for a's slices
       k_split32<<<eg, 256, 0, st>>>(wv.dev, b.Fc, b.Y[0], b.Y[1]);
       SM_KCHECK();
@@ -1522,10 +1441,7 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
       // C = M S (symmetric to first order) -> CG residual
       TcGemmParams g4 = tc(SYM, NSYM, MS_YH, MS_YL, c_hi, c_lo, 1, 1.0f, 0.0f);
       g4.out_f32 = b.cr;
-      g4.upper_only = 1;
       SM_CUDA(launch(g4));
-      k_mirror_f32<<<pair_grid_stream(wv), dim3(8, 32), 0, st>>>(wv.dev, b.cr);
-      SM_KCHECK();
       // CG on L -> H L + L H, per submatrix until the relative residual is below cg_tol
       SM_CUDA(cudaMemsetAsync(rr, 0, sizeof(double) * 4 * max_wave, st));
       SM_CUDA(cudaMemsetAsync(ms->cg_done, 0, sizeof(int) * max_wave, st));
@@ -1844,7 +1760,6 @@ submat_status Plan::backward_wave_tc(size_t wi, const double* K, double mu, cons
     p.skip_state = -1;
     p.alpha = 1.0f; p.beta = 0.0f; p.diag = 0.0f;
     p.sym = sym;
-    p.upper_only = sym;  // symmetric results: upper tiles, then a mirror pass
     p.flags = d_flags;
     p.timeout_cycles = tmo;
     return p;
@@ -1887,8 +1802,6 @@ submat_status Plan::backward_wave_tc(size_t wi, const double* K, double mu, cons
       g1.out_hi = P[AS_ZH]; g1.out_lo = P[AS_ZL];
       if (extra < 0) g1.res2 = ns.res2;
       SM_CUDA(launch(g1));
-      k_mirror_split<<<pg, dim3(8, 32), 0, st>>>(wv.dev, P[AS_ZH], P[AS_ZL], nullptr, 0);
-      SM_KCHECK();
       if (k == 0 && opt.beta_mode == 0) {  // as in the forward path; E_0 and E_0^T follow X_0
         const CertSquare sq{2, P[AS_ZH], P[AS_ZL], g1.alpha, g1.diag};
         const CertLinear lin{3, {P[AS_X0H], P[AS_E0H], P[AS_TH]}, {P[AS_X0L], P[AS_E0L], P[AS_TL]}};
@@ -1932,8 +1845,6 @@ submat_status Plan::backward_wave_tc(size_t wi, const double* K, double mu, cons
       g2.out_hi = P[xn]; g2.out_lo = P[xn + 1];
       SM_CUDA(launch(g2));
       ++updates;
-      k_mirror_split<<<pg, dim3(8, 32), 0, st>>>(wv.dev, P[xn], P[xn + 1], nullptr, 0);
-      SM_KCHECK();
       k_transpose_split<<<pg, dim3(8, 32), 0, st>>>(wv.dev, P[en], P[en + 1], P[AS_TH], P[AS_TL]);
       SM_KCHECK();
       if (extra < 0) {

@@ -13,8 +13,8 @@
 //
 // Roles (192 or 320 threads): warp 0 issues TMA loads, warp 1 owns TMEM and one of
 // its lanes issues the MMAs, warps 2-5 (or 2-9) drain the accumulator (one TMEM
-// lane quarter each, or half of one) and write the tile -- and, for symmetric outputs, its mirror
-// through a shared-memory transpose.  Every mbarrier wait is bounded; on
+// lane quarter each, or half of one) and write the tile -- and, for symmetric
+// outputs, its mirror.  Every mbarrier wait is bounded; on
 // timeout the kernel raises FLAG_TIMEOUT, drains its own copies and MMAs,
 // frees TMEM and returns.
 #include <cuda.h>
@@ -34,12 +34,10 @@ namespace {
 
 constexpr int BM = 128, BK = 64;
 constexpr int TILE_BYTES = BM * BK * 2;  // one 128 x 64 BF16 operand tile (A side)
-constexpr int STG_PITCH = 33;            // staged row pitch (32-bit words)
 // integer outputs: one 16-column int64 row segment per thread, rows 144 bytes
-// apart (16-byte aligned for the bulk copy, padded against bank conflicts);
-// the buffer doubles as the 32-bit transpose stage of the mirror
+// apart (16-byte aligned for the bulk copy, padded against bank conflicts)
 constexpr int I64_SEG = 16, I64_PITCH = 144;
-constexpr int STG_BYTES = (BM * I64_PITCH > BM * STG_PITCH * 4) ? BM * I64_PITCH : BM * STG_PITCH * 4;
+constexpr int STG_BYTES = BM * I64_PITCH;
 
 // instruction descriptor: D F32, A and B BF16, both K-major, M = 128, N = cols
 // (FP16 operands clear the two format fields, bits 7-9 and 10-12)
@@ -123,19 +121,18 @@ __device__ __forceinline__ void store_row(const TcGemmParams& p, int64_t idx, co
   }
 }
 
-// store o[q] for q in [q_lo, q_hi) only (diagonal tiles of symmetric outputs):
-// whole segments as vectors, element stores only where the diagonal crosses
+// store o[q] for q >= q_lo only (diagonal tiles of symmetric outputs): whole
+// segments as vectors, element stores only where the diagonal crosses
 template <bool F16>
-__device__ __forceinline__ void store_range(const TcGemmParams& p, int64_t idx, const float* o,
-                                            int q_lo, int q_hi) {
-  if (q_lo >= 32 || q_hi <= 0 || q_lo >= q_hi) return;
-  if (q_lo <= 0 && q_hi >= 32) {
+__device__ __forceinline__ void store_range(const TcGemmParams& p, int64_t idx, const float* o, int q_lo) {
+  if (q_lo >= 32) return;
+  if (q_lo <= 0) {
     store_row<F16>(p, idx, o);
     return;
   }
 #pragma unroll
   for (int q = 0; q < 32; ++q) {
-    if (q < q_lo || q >= q_hi) continue;
+    if (q < q_lo) continue;
     if (p.out_f32) {
       p.out_f32[idx + q] = o[q];
     } else {
@@ -188,17 +185,50 @@ __device__ __forceinline__ void load_c0(const TcGemmParams& p, int64_t idx, floa
   }
 }
 
-// The epilogue a launch compiles in (the host checks what each needs):
-// EPI_GENERAL anything, the tile's 128 columns live in registers; EPI_FLOAT one
-// accumulator, a 16-bit pair or FP32 output, no mirror, double-buffered TMEM;
-// EPI_INT integer sums of slice products.  The last two drain 32 columns at a
-// time.
-// EPI_FLOAT has eight epilogue warps, two for each TMEM lane quarter, which take
-// the chunks in turn: with four, converting and storing a tile of few k-blocks
-// took longer than its MMAs (1000 FP16 products of 192 dims: 129 -> 111 us, and
-// 83 us at a width of 256).
-enum Epilogue { EPI_GENERAL, EPI_FLOAT, EPI_INT };
+// The epilogue a launch compiles in, both draining 32 columns at a time:
+// EPI_FLOAT one accumulator, a 16-bit pair or FP32 output, double-buffered TMEM;
+// EPI_INT integer sums of slice products.
+// EPI_FLOAT has eight warps, two for each TMEM lane quarter, which take the
+// chunks in turn (with four, a tile of few k-blocks took longer to convert and
+// store than its MMAs: 1000 FP16 products of 192 dims 129 -> 111 us, and 83 us at
+// a width of 256).  They write the mirror of a symmetric result too, so that no
+// pass reads it back: 700 submatrices of 504-704 dims 51.4 -> 48.7 ms a build.
+enum Epilogue { EPI_FLOAT, EPI_INT };
 __host__ __device__ constexpr int epi_warps(int mode) { return mode == EPI_FLOAT ? 8 : 4; }
+
+// A warp's 32 x 32 chunk (lane: row, o: columns) to its mirrored place, whose
+// first row and column are row0 and col0; diagonal: only entries below the
+// diagonal.  FP32 goes out column by column; of a 16-bit pair two lanes exchange
+// halves, so that each stores two rows' entries of one column as a word.  (Not
+// through shared memory, whose bandwidth bounds the MMAs: a staged transpose
+// made Newton-Schulz products 30 % longer.)
+template <bool F16>
+__device__ __forceinline__ void store_mirror(const TcGemmParams& p, int64_t base, int ld, int row0, int col0,
+                                             const float* o, int lane, bool diagonal) {
+  if (p.out_f32) {
+    float* d = p.out_f32 + base + int64_t(row0) * ld + col0 + lane;
+#pragma unroll
+    for (int q = 0; q < 32; ++q)
+      if (!diagonal || q > lane) d[int64_t(q) * ld] = o[q];
+    return;
+  }
+  const int odd = lane & 1, c = lane & ~1;
+  const int64_t idx = base + int64_t(row0 + odd) * ld + col0 + c;
+  auto put = [&](__nv_bfloat16* out, int64_t i, uint32_t v, int r) {
+    if (!diagonal || r > c + 1) *reinterpret_cast<uint32_t*>(out + i) = v;
+    else if (r == c + 1) out[i] = __ushort_as_bfloat16(static_cast<unsigned short>(v & 0xFFFFu));
+  };
+#pragma unroll
+  for (int q = 0; q < 32; q += 2) {
+    uint32_t hw, lw;
+    if constexpr (F16) pack_split2_h(o[q], o[q + 1], &hw, &lw);
+    else pack_split2(o[q], o[q + 1], &hw, &lw);
+    const uint32_t ph = __shfl_xor_sync(0xffffffffu, hw, 1), pl = __shfl_xor_sync(0xffffffffu, lw, 1);
+    const int64_t i = idx + int64_t(q) * ld;
+    put(p.out_hi, i, odd ? __byte_perm(ph, hw, 0x7632) : __byte_perm(hw, ph, 0x5410), q + odd);
+    if (p.out_lo) put(p.out_lo, i, odd ? __byte_perm(pl, lw, 0x7632) : __byte_perm(lw, pl, 0x5410), q + odd);
+  }
+}
 
 // hi + lo += x, both FP32, with the rounding error kept
 __device__ __forceinline__ void add_pair(float x, float& hi, float& lo) {
@@ -210,7 +240,6 @@ __device__ __forceinline__ void add_pair(float x, float& hi, float& lo) {
 template <int BN, int MODE, bool F16>
 __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const __grid_constant__ TcGemmParams p) {
   constexpr int TILE_B = BN * BK * 2;  // one BN x 64 BF16 operand tile (B side)
-  constexpr bool LEAN = MODE != EPI_GENERAL;
   constexpr int HALVES = BN / 128;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -387,12 +416,11 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const 
       const int n = p.n[s];
       const int64_t base = p.off[s];
       const int rg = item.y * BM + r;
-      double part = 0.0;
       const uint32_t tbase = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(ab * p.nacc * BN);
       // 32 columns at a time, so only one chunk is live in registers, and the
       // diagonal handled only on diagonal sub-tiles.  TMEM is released after its
       // last read.
-      if constexpr (LEAN) {
+      {
         if constexpr (MODE == EPI_INT) {
           // exact integer sums of slice products (full tiles): per 32-column
           // chunk the sum over the accumulators of acc_k * 2^shift_k in 64-bit
@@ -492,8 +520,10 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const 
             }
             if (p.res2) add_pair(p.sym && !diag_sym ? 2.0f * pr : pr, ph, pl);
             if (p.dot_c0) add_pair(2.0f * pd, ph, pl);
-            if (diag_sym) store_range<F16>(p, idx, o, r - c * 32, 32);
+            if (diag_sym) store_range<F16>(p, idx, o, r - c * 32);
             else store_row<F16>(p, idx, o);
+            if (!p.sym || (diag_sym && c < quarter)) continue;
+            store_mirror<F16>(p, base, ld, cg0, item.y * BM + quarter * 32, o, lane, diag_sym && c == quarter);
           }
           // FP64 instructions hold their pipe for 64 clocks: sums stay in FP32
           // pairs up to one conversion per warp
@@ -510,156 +540,10 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const 
             }
           }
         }
-      } else {
-      for (int h = 0; h < HALVES; ++h) {
-      float acc[128];
-      const uint32_t tb = tbase + uint32_t(h * 128);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) tmem_ld32(tb + uint32_t(c * 32), acc + c * 32);
-      tmem_wait_ld();
-      if (p.out_i64 && p.nacc == 2) {
-        // two exact integer accumulators of adjacent levels: acc0 * 2^d + acc1
-        // (|acc| < 2^24, d <= 6: the sum fits in 31 bits), kept as int bits
-        float tmp[32];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          tmem_ld32(tb + uint32_t(BN + c * 32), tmp);
-          tmem_wait_ld();
-#pragma unroll
-          for (int q = 0; q < 32; ++q)
-            acc[c * 32 + q] = __int_as_float(__float2int_rn(acc[c * 32 + q]) * (1 << p.i64_dshift) +
-                                             __float2int_rn(tmp[q]));
-        }
-      } else {
-        for (int a = 1; a < p.nacc; ++a) {
-          float tmp[32];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            tmem_ld32(tb + uint32_t(a * BN + c * 32), tmp);
-            tmem_wait_ld();
-#pragma unroll
-            for (int q = 0; q < 32; ++q) acc[c * 32 + q] += tmp[q];
-          }
-        }
-      }
-      if (h == HALVES - 1) {
-        tc_fence_before();
-        if (!p.test_skip_arrive) mbar_arrive(&tempty[ab]);
-      }
-      // this half is the 128 x 128 sub-tile (item.y, sub_tj) of C
-      const int sub_tj = item.z * HALVES + h;
-      // symmetric output: sub-tiles below the diagonal are not written, those
-      // above it are mirrored, diagonal ones keep their upper triangle and take
-      // the strict lower one from it, so C is exactly symmetric whatever the
-      // accumulation order
-      if (p.sym && sub_tj < item.y) continue;
-      const bool diag_sym = p.sym && item.y == sub_tj;
-      const bool mirror = p.sym != 0 && !p.upper_only;
-      const double res_weight = (p.sym && !diag_sym) ? 2.0 : 1.0;  // the mirror counts too
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int cg0 = sub_tj * 128 + c * 32;
-        float o[32];
-        const bool inside = (rg < ld) && (cg0 < ld);
-        if (p.out_i64) {
-          // exact integer sums of slice products, accumulated in 64-bit integers
-          // (full tiles only: no mirror, no diagonal mask).  Each 16-column row
-          // segment is staged in shared memory and handed to a bulk copy (first
-          // product) or a bulk add in L2 (later ones): no loads on the SM.
-          if (inside) {
-            const long long mul = 1LL << p.i64_shift;
-            uint8_t* srow = reinterpret_cast<uint8_t*>(stg) + r * I64_PITCH;
-#pragma unroll
-            for (int seg = 0; seg < 32 / I64_SEG; ++seg) {
-              // the previous bulk operation of this thread has read its source
-              asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-#pragma unroll
-              for (int q = 0; q < I64_SEG; ++q) {
-                const float x = acc[c * 32 + seg * I64_SEG + q];
-                const long long v = (long long)(p.nacc == 2 ? __float_as_int(x) : __float2int_rn(x)) * mul;
-                *reinterpret_cast<long long*>(srow + 8 * q) = v;
-              }
-              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-              long long* d = p.out_i64 + base + int64_t(rg) * ld + cg0 + seg * I64_SEG;
-              if (p.i64_accumulate)
-                asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.u64 [%0], [%1], %2;" ::"l"(d),
-                             "r"(smem_u32(srow)), "n"(I64_SEG * 8)
-                             : "memory");
-              else
-                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(d),
-                             "r"(smem_u32(srow)), "n"(I64_SEG * 8)
-                             : "memory");
-              asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-            }
-          }
-          continue;
-        }
-        if (inside) {
-          float c0[32];
-          const int64_t idx = base + int64_t(rg) * ld + cg0;
-          const bool has_c0 = (p.c0_f32 || p.c0_hi) && p.beta != 0.0f && !p.dot_c0;
-          if (has_c0 || p.dot_c0) load_c0<F16>(p, idx, c0);
-          const int dq = (rg < n) ? rg - cg0 : -1;  // diagonal position in this segment
-#pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            float v = p.alpha * acc[c * 32 + q];
-            if (has_c0) v = fmaf(p.beta, c0[q], v);
-            if (q == dq) v += p.diag;
-            o[q] = v;
-          }
-          if (p.dot_c0) {
-            float pc = 0.0f;
-#pragma unroll
-            for (int q = 0; q < 32; ++q) pc = fmaf(o[q], c0[q], pc);
-            part += 2.0 * double(pc);
-          }
-          if (p.res2) {
-            float pc = 0.0f;
-#pragma unroll
-            for (int q = 0; q < 32; ++q) {
-              const int cg = cg0 + q;
-              const float e = acc[c * 32 + q] - ((rg == cg && rg < n) ? 1.0f : 0.0f);
-              pc = fmaf(e, e, pc);
-            }
-            part += res_weight * double(pc);
-          }
-          if (diag_sym) store_range<F16>(p, idx, o, r - c * 32, 32);
-          else store_row<F16>(p, idx, o);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 32; ++q) o[q] = 0.0f;
-        }
-        if (mirror) {
-          // transpose the 128 x 32 chunk through shared memory; column q of
-          // row r sits at q ^ 8 (r / 32), so that the row writes and the column
-          // reads below both hit 32 distinct banks
-#pragma unroll
-          for (int q = 0; q < 32; ++q) stg[r * STG_PITCH + (q ^ (8 * quarter))] = __float_as_uint(o[q]);
-          epi_bar();
-          const int t = threadIdx.x - 64;
-          const int q = t >> 2, part4 = t & 3;
-          const int mrow = sub_tj * 128 + c * 32 + q;       // row of the mirrored tile
-          const int mcol0 = item.y * BM + part4 * 32;      // its first column
-          if (mrow < ld && mcol0 < ld) {
-            float w[32];
-#pragma unroll
-            for (int i = 0; i < 32; ++i) w[i] = __uint_as_float(stg[(part4 * 32 + i) * STG_PITCH + (q ^ (8 * part4))]);
-            if (diag_sym) store_range<F16>(p, base + int64_t(mrow) * ld + mcol0, w, 0, c * 32 + q - part4 * 32);
-            else store_row<F16>(p, base + int64_t(mrow) * ld + mcol0, w);
-          }
-          epi_bar();
-        }
-      }
-      }  // halves
-      }  // general epilogue
-      if (!LEAN && (p.res2 || p.dot_c0)) {
-#pragma unroll
-        for (int o2 = 16; o2 > 0; o2 >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o2);
-        if (lane == 0 && part != 0.0) atomicAdd(p.res2 ? &p.res2[s] : &p.dot_c0[s], part);
       }
     }
     // bulk copies and adds issued by this thread are complete and visible
-    if (p.out_i64) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if constexpr (MODE == EPI_INT) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
   __syncthreads();
   if (warp == 1) {
@@ -689,39 +573,28 @@ cudaError_t launch_tc_gemm(const TcGemmParams& p, int grid, cudaStream_t st) {
   if (bn == 256 && (p.tmem_cols != 512 || !(p.nacc == 1 || (p.nacc == 2 && p.out_i64))))
     return cudaErrorInvalidValue;
   if (p.nacc * bn > p.tmem_cols) return cudaErrorInvalidValue;
-  if (p.out_i64 && p.sym) return cudaErrorInvalidValue;  // integer outputs: full tiles only
-  // the lean epilogue combines up to four integer accumulators in 64 bits
-  // (weights 2^i64_shifts[k]); the general one two in 32 bits (d <= 6)
-  const bool lean_i64 = p.out_i64 && !p.sym && p.nacc <= 4 && p.nacc * bn <= p.tmem_cols &&
-                        (p.nacc > 2 ? bn == 128 : p.tmem_cols >= 2 * p.nacc * bn);
-  if (p.out_i64 && !lean_i64 && (p.nacc > 2 || (p.nacc == 2 && (p.i64_dshift < 0 || p.i64_dshift > 6))))
-    return cudaErrorInvalidValue;
-  if (p.out_i64)
+  if (p.out_i64) {
+    // full tiles; up to four accumulators of weights 2^i64_shifts[k], combined in 64 bits
+    if (p.sym || p.f16 || p.nacc > 4 || (p.nacc > 2 ? bn != 128 : p.tmem_cols < 2 * p.nacc * bn))
+      return cudaErrorInvalidValue;
     for (int k = 0; k < p.nacc; ++k)
-      if (lean_i64 && (p.i64_shifts[k] < 0 || p.i64_shifts[k] > 36)) return cudaErrorInvalidValue;
+      if (p.i64_shifts[k] < 0 || p.i64_shifts[k] > 36) return cudaErrorInvalidValue;
+  } else if (p.nacc != 1 || p.tmem_cols < 2 * bn || !(p.out_f32 || p.out_hi)) {
+    return cudaErrorInvalidValue;
+  }
   const int smem = tc_smem_bytes(p.na, p.nb, p.nstage, bn);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  // the lean epilogue: one accumulator, double-buffered in TMEM, BF16-pair or
-  // FP32 output without a mirror
-  const bool lean = (p.out_i64 ? lean_i64
-                                : p.tmem_cols >= 2 * bn && p.nacc == 1 && !(p.sym && !p.upper_only) &&
-                                      (p.out_f32 || p.out_hi));
   auto run = [&](auto kern, int mode) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, 64 + 32 * epi_warps(mode), smem, st>>>(p);
     return cudaSuccess;
   };
-  // FP16 operands: lean launches only (the Newton-Schulz products)
-  if (p.f16 && !lean) return cudaErrorInvalidValue;
-  if (p.f16 && p.out_i64) return cudaErrorInvalidValue;
   cudaError_t e;
   auto pick = [&](auto width) -> cudaError_t {
     constexpr int W = decltype(width)::value;
-    if (p.f16) return run(k_tc_gemm<W, EPI_FLOAT, true>, EPI_FLOAT);
-    if (!lean) return run(k_tc_gemm<W, EPI_GENERAL, false>, EPI_GENERAL);
     if (p.out_i64) return run(k_tc_gemm<W, EPI_INT, false>, EPI_INT);
-    return run(k_tc_gemm<W, EPI_FLOAT, false>, EPI_FLOAT);
+    return p.f16 ? run(k_tc_gemm<W, EPI_FLOAT, true>, EPI_FLOAT) : run(k_tc_gemm<W, EPI_FLOAT, false>, EPI_FLOAT);
   };
   e = bn == 256 ? pick(std::integral_constant<int, 256>()) : pick(std::integral_constant<int, 128>());
   if (e != cudaSuccess) return e;

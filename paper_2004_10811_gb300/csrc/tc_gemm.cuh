@@ -37,8 +37,7 @@ struct TcGemmParams {
   // a BF16 (hi, lo) split
   float alpha, beta, diag;
   int sym;                        // symmetric result: items have ti <= tj; the mirrored tile is
-                                  // written too unless upper_only (then a separate pass copies it)
-  int upper_only;
+                                  // written too
   float* out_f32;
   __nv_bfloat16* out_hi;
   __nv_bfloat16* out_lo;          // may be null: plain BF16 output
@@ -48,15 +47,10 @@ struct TcGemmParams {
   double* res2;                   // optional ||acc - I_n||_F^2 per submatrix (before alpha, beta, diag)
   double* dot_c0;                 // optional: 2 <C, C0> per submatrix (C0 = c0_f32, beta unused)
   // Exact integer output (sliced products, full tiles only): with out_i64 set,
-  // the tile value is the integer accumulator times 2^i64_shift, written or
-  // (i64_accumulate) added to out_i64; row/column scales are applied later.
-  // With nacc = 2 the two accumulators hold adjacent levels: the tile value
-  // is (acc0 * 2^i64_dshift + acc1) * 2^i64_shift, 0 <= i64_dshift <= 6.
+  // the tile value is the sum of the integer accumulators times 2^i64_shifts[k],
+  // up to four of any weights, written or (i64_accumulate) added to out_i64;
+  // row/column scales are applied later.
   long long* out_i64;
-  int i64_shift;
-  int i64_dshift;
-  // lean epilogue: accumulator k carries the weight 2^i64_shifts[k] and up to
-  // four accumulators are combined in 64-bit integers (any weights)
   int i64_shifts[4];
   int i64_accumulate;
   // operand and pair format: 0 BF16, 1 FP16 (A and B always share one
