@@ -871,11 +871,19 @@ int sym256_count(int t128, int t256) {
   return c;
 }
 
+// Blocks a submatrix gets of `units` units of work: `per` units each, few and
+// long, but fewer where the wave would give less than four blocks per SM (32
+// submatrices of 132-174 dims: 96 blocks of k_comm; with this and narrower GEMM
+// tiles there 1.42 -> 1.28 ms a build)
+unsigned blocks_for(const Wave& wv, int64_t units, int64_t per, int64_t most) {
+  const int64_t want = 4 * int64_t(num_sms());
+  while (per > 1 && (units + per - 1) / per * wv.count < want) per /= 2;
+  return unsigned(std::max<int64_t>(1, std::min<int64_t>((units + per - 1) / per, most)));
+}
+
 dim3 elem_grid(const Wave& wv) {
-  // about 32 entries per thread: few, long blocks
-  int64_t bx = (wv.max_ld2 + 256 * 32 - 1) / (256 * 32);
-  bx = std::max<int64_t>(1, std::min<int64_t>(bx, 256));
-  return dim3(unsigned(bx), unsigned(wv.count));
+  // 256 threads of about 32 entries, four at a time
+  return dim3(blocks_for(wv, (wv.max_ld2 + 1023) / 1024, 8, 256), unsigned(wv.count));
 }
 
 dim3 pair_grid(const Wave& wv) {
@@ -889,10 +897,8 @@ dim3 pair_grid(const Wave& wv) {
 // eight pairs per block, so that blocks are few and long enough for their
 // launch cost to vanish against their traffic.
 dim3 pair_grid_stream(const Wave& wv) {
-  int64_t t = 1;
-  for (int64_t l : wv.bucket_ld) t = std::max<int64_t>(t, l / 32);
-  int64_t np = t * (t + 1) / 2;
-  return dim3(unsigned(std::max<int64_t>(1, std::min<int64_t>((np + 7) / 8, 512))), unsigned(wv.count));
+  const int64_t t = max_ld(wv) / 32;
+  return dim3(blocks_for(wv, t * (t + 1) / 2, 8, 512), unsigned(wv.count));
 }
 
 struct MixedState {
@@ -1209,7 +1215,7 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
     // split products of the correction: 256-wide tiles (measured 12 % faster
     // per launch than 128 on the 1024x23 workload); the sliced products pick
     // their own width below
-    use_width(opt.tile_n_corr ? opt.tile_n_corr : 256);
+    use_width(opt.tile_n_corr ? opt.tile_n_corr : (wv.n_full256 >= 2 * nsm ? 256 : 128));
     std::vector<int> lp_iters(wv.count);
     SM_CUDA(cudaMemcpyAsync(lp_iters.data(), ns.iters, sizeof(int) * wv.count, cudaMemcpyDeviceToHost, st));
     SM_CUDA(cudaMemsetAsync(ms->cg_count, 0, sizeof(int) * max_wave, st));
@@ -1236,7 +1242,7 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
     SlicePtrs sl_s{{b.X[0][0], b.X[0][1], b.X[1][0], b.X[1][1], b.Y[0], b.Y[1]}};
     SlicePtrs sl_a{{b.Ah[0], b.Ah[1], b.Hh[0], b.Hh[1], b.Z[0], b.Z[1]}};
     // about eight rows per warp (k_slice takes one row per warp at a time)
-    const dim3 slice_grid(unsigned(std::max<int64_t>(1, std::min<int64_t>(max_ld / 64, 256))), unsigned(wv.count));
+    const dim3 slice_grid(blocks_for(wv, max_ld / 8, 8, 256), unsigned(wv.count));
     // C (+)= sign * X Y^T from the slices: level t = p + q weighs 2^(-6 t); each
     // launch sums at most per_acc products of one level in one exact accumulator
     // slice products issued (all residual products, this wave): over 128 x 128
