@@ -53,25 +53,32 @@ namespace submat {
 // discrete cosine transform of the first kind; exact for degree < N).
 // cos(k theta_n) = cos(pi j / (2N)) with j = k (2n + 1) mod 4N, read from a
 // table, so no rounding accumulates with k.
-static void cheb_coefficients(double c, int N, int ncoef, std::vector<double>* out) {
+static submat_status cheb_coefficients(double c, int N, int ncoef, std::vector<double>* out,
+                                       const ChebTransform& transform) {
   const int64_t P = 4 * int64_t(N);
   std::vector<double> cosv(static_cast<size_t>(P)), g(static_cast<size_t>(N));
   for (int64_t j = 0; j < P; ++j) cosv[size_t(j)] = std::cos(M_PI * double(j) / (2.0 * N));
   for (int n = 0; n < N; ++n) g[n] = std::tanh(c * cosv[size_t(2 * n + 1)]);
   out->assign(ncoef, 0.0);
-  for (int k = 0; k < ncoef; ++k) {
-    double acc = 0.0;
-    int64_t j = k, step = 2 * int64_t(k) % P;  // j = k (2n + 1) mod 4N
-    for (int n = 0; n < N; ++n) {
-      acc += g[n] * cosv[size_t(j)];
-      j += step;
-      if (j >= P) j -= P;
+  if (transform) {
+    SM_TRY(transform(g, cosv, ncoef, out->data()));
+  } else {
+    for (int k = 0; k < ncoef; ++k) {
+      double acc = 0.0;
+      int64_t j = k, step = 2 * int64_t(k) % P;  // j = k (2n + 1) mod 4N
+      for (int n = 0; n < N; ++n) {
+        acc += g[n] * cosv[size_t(j)];
+        j += step;
+        if (j >= P) j -= P;
+      }
+      (*out)[k] = acc;
     }
-    (*out)[k] = (k == 0 ? 1.0 : 2.0) * acc / N;
   }
+  for (int k = 0; k < ncoef; ++k) (*out)[k] = (k == 0 ? 1.0 : 2.0) * (*out)[k] / N;
+  return SUBMAT_OK;
 }
 
-submat_status fermi_poly(double c, double tol, int max_degree, FermiPoly* out) {
+submat_status fermi_poly(double c, double tol, int max_degree, FermiPoly* out, const ChebTransform& transform) {
   if (!(c > 0.0) || !std::isfinite(c)) {
     set_error("finite temperature: bad scale c = %g", c);
     return SUBMAT_ERR_INVALID_ARG;
@@ -83,7 +90,7 @@ submat_status fermi_poly(double c, double tol, int max_degree, FermiPoly* out) {
   double tail = 0.0;
   for (int N = 256;; N *= 2) {
     const int ncoef = N / 2;
-    cheb_coefficients(c, N, ncoef, &coef);
+    SM_TRY(cheb_coefficients(c, N, ncoef, &coef, transform));
     // coefficients below the rounding floor of the transform are noise, not
     // truncation: the series counts up to the last one above it
     double cmax = 0.0;
@@ -150,6 +157,26 @@ int fermi_clenshaw_exponent(const FermiPoly& P) {
 }
 
 namespace {
+
+// sums[k] = sum_n g_n cos(k theta_n), one thread per k in ascending n, as the host
+// does.  The N^2 / 2 terms took the host 10 ms an evaluation at degree ~400 (N =
+// 2048), a third of it; here a chain of N multiply-adds per warp, spread over the
+// SMs, takes ~0.1 ms: FP32 mu search 171.3 -> 120.4 ms, FP64 build 28.3 -> 26.4.
+__global__ void __launch_bounds__(32) k_cheb_sums(int N, int ncoef, const double* __restrict__ g,
+                                                  const double* __restrict__ cosv, double* __restrict__ sums) {
+  const int k = blockIdx.x * 32 + threadIdx.x;
+  if (k >= ncoef) return;
+  const int P = 4 * N, step = 2 * k;  // j = k (2n + 1) mod 4N; 2k < 4N
+  int j = k;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int n = 0; n < N; ++n) {
+    acc = fma(g[n], cosv[j], acc);
+    j += step;
+    if (j >= P) j -= P;
+  }
+  sums[k] = acc;
+}
 
 // X <- r_s X and T2 <- r_s^2 (T2 + I) - I (the square rescaled), r_s = ratio[s]
 template <typename T>
@@ -270,6 +297,24 @@ size_t fermi_dual_bytes_per_elem(int prec) {
   return 8 + size_t(2 * kFermiBuffers) * (prec == SUBMAT_FP64 ? 8 : 4);
 }
 
+submat_status Plan::cheb_transform(const std::vector<double>& g, const std::vector<double>& cosv, int ncoef,
+                                   double* sums, cudaStream_t st) {
+  const size_t N = g.size(), need = N + cosv.size() + size_t(ncoef);
+  if (need > cheb_cap) {  // kept by the plan; a larger N than before is rare
+    SM_TRY(alloc(&d_cheb, need, "Chebyshev transform"));
+    cheb_cap = need;
+  }
+  double* dc = d_cheb + N;
+  double* ds = dc + cosv.size();
+  SM_CUDA(cudaMemcpyAsync(d_cheb, g.data(), 8 * N, cudaMemcpyHostToDevice, st));
+  SM_CUDA(cudaMemcpyAsync(dc, cosv.data(), 8 * cosv.size(), cudaMemcpyHostToDevice, st));
+  k_cheb_sums<<<(ncoef + 31) / 32, 32, 0, st>>>(int(N), ncoef, d_cheb, dc, ds);
+  SM_KCHECK();
+  SM_CUDA(cudaMemcpyAsync(sums, ds, 8 * size_t(ncoef), cudaMemcpyDeviceToHost, st));
+  SM_CUDA(cudaStreamSynchronize(st));
+  return SUBMAT_OK;
+}
+
 // One wave.  Forward: D = (I - p(X)) / 2 on the extracted columns, with the
 // trace and sum-of-squares partials for dN/dmu.  With Dbar (the adjoint):
 // every matrix M of the evaluation carries a derivative part M' (dual
@@ -381,7 +426,10 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
     SM_KCHECK();
   }
   FermiPoly P;
-  SM_TRY(fermi_poly(sigma / (2.0 * opt.kT), tol_poly, kFermiMaxDegree, &P));
+  SM_TRY(fermi_poly(sigma / (2.0 * opt.kT), tol_poly, kFermiMaxDegree, &P,
+                    [&](const std::vector<double>& g, const std::vector<double>& cosv, int ncoef, double* sums) {
+                      return cheb_transform(g, cosv, ncoef, sums, st);
+                    }));
   fermi_degree = std::max(fermi_degree, P.m);
   fermi_trunc = std::max(fermi_trunc, P.trunc);
   T* out = nullptr;

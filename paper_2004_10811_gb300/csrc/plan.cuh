@@ -77,7 +77,12 @@ struct FermiPoly {
 // Exponent e with |b_j(x)| <= 2^e on [-1, 1] for every Clenshaw term b_j of P
 // and p, 0 at least.
 int fermi_clenshaw_exponent(const FermiPoly& P);
-submat_status fermi_poly(double c, double tol, int max_degree, FermiPoly* out);
+// A transform turns the N node values g and cos(pi j / (2N)), j < 4N, into the
+// first ncoef coefficients times N / 2 (N for k = 0); null: on the host.
+using ChebTransform = std::function<submat_status(const std::vector<double>& g, const std::vector<double>& cosv,
+                                                  int ncoef, double* sums)>;
+submat_status fermi_poly(double c, double tol, int max_degree, FermiPoly* out,
+                         const ChebTransform& transform = ChebTransform());
 size_t fermi_bytes_per_elem(int prec);
 
 struct Wave {
@@ -204,6 +209,8 @@ struct Plan {
   // finite temperature: per block column sum of squares of the extracted
   // columns, and the last evaluation's polynomial
   double* d_sqpart = nullptr;
+  double* d_cheb = nullptr;  // node values, cosines and sums of the Chebyshev transform
+  size_t cheb_cap = 0;       // its entries
   int fermi_degree = 0;
   double fermi_trunc = 0.0, fermi_flops = 0.0;
 
@@ -256,6 +263,8 @@ struct Plan {
   template <typename T>
   submat_status fermi_wave(Wave& wv, int wi, const double* K, double mu, double* D, const double* Dbar, double* Kbar,
                            void* w, int64_t E, cudaStream_t st);
+  submat_status cheb_transform(const std::vector<double>& g, const std::vector<double>& cosv, int ncoef, double* sums,
+                               cudaStream_t st);
   submat_status fermi_dn_dmu(cudaStream_t st, double* out);
   submat_status backward_fermi(const double* K, double mu, const double* Dbar, double* Kbar, double* dN_dmu,
                                cudaStream_t st);
