@@ -498,7 +498,8 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
 // b_j 2^-e (fermi_clenshaw_exponent).  Residue set 0 holds the factor that
 // stays (T_2, then Y), set 1 the one that each pass renews.
 // 720 submatrices of 240 molecules (13 + 5 + 5 functions, 6.5 A, kT 0.05): a
-// build took 573 ms with the FP64 SIMT GEMM and takes 28.3 ms.
+// build took 573 ms with the FP64 SIMT GEMM and takes 24.9 ms, 10.5 of them in
+// the giant steps' passes (k_rns_cheb).
 submat_status Plan::fermi_rns(int wi, const FermiPoly& P, double** out, int* products, cudaStream_t st) {
   constexpr int H = kFermiBaby / 2;
   static_assert(H == RNS_COMB, "one coefficient per stored odd T_k");
@@ -546,7 +547,7 @@ submat_status Plan::fermi_rns(int wi, const FermiPoly& P, double** out, int* pro
   c.R = R[1];
   for (int j = P.blocks - 1; j >= 0; --j) {
     long long* W = bb[j & 1];  // b_{j+2}'s place
-    for (int q = 0; q < H; ++q) c.coef[q] = std::llrint(std::ldexp(P.r[size_t(j) * H + q], 60 - e));
+    for (int q = 0; q < H; ++q) c.coef[q] = std::llrint(std::ldexp(P.r[size_t(j) * H + q], RNS_FRAC - e));
     if (j < P.blocks - 1) {
       SM_TRY(product());
       c.F = F;

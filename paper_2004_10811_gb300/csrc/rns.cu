@@ -626,11 +626,21 @@ __global__ void __launch_bounds__(256) k_rns_cheb2(WaveDev w, const long long* _
   }
 }
 
+// t c = 2^64 h + 2^32 m to a few 2^32, summed over the terms, from balanced
+// 32-bit halves: |t| <= 2^58 and |c| < 2^60 keep the sums of RNS_COMB terms in range
+__device__ __forceinline__ void add_product(long long t, long long c, long long& h, long long& m) {
+  const int tl = int(t), th = int(t >> 32) - (tl >> 31);
+  const int cl = int(c), ch = int(c >> 32) - (cl >> 31);
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(h) : "r"(th), "r"(ch));
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(m) : "r"(th), "r"(cl));
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(m) : "r"(tl), "r"(ch));
+  m += __mulhi(tl, cl);
+}
+
 // One step of the recurrences, as a pass over tile pairs: bound by memory
 // traffic (the residues written, 28 bytes an entry, are the largest part), so
 // the combination of the stored odd T_k is formed here instead of in a pass of
-// its own, and only upper tiles are read.  Its 64-bit upper halves are floors:
-// RNS_COMB / 2 restores their mean (where they are floors of anything but 0).
+// its own, and only upper tiles are read.
 template <bool COMB>
 __global__ void __launch_bounds__(256) k_rns_cheb(WaveDev w, const __grid_constant__ RnsCheb p) {
   __shared__ long long v[64][PITCH];
@@ -659,17 +669,15 @@ __global__ void __launch_bounds__(256) k_rns_cheb(WaveDev w, const __grid_consta
         x.y -= z.y;
       }
       if constexpr (COMB) {
-        longlong2 any = make_longlong2(0, 0);
+        long long hx = 0, mx = 0, hy = 0, my = 0;
 #pragma unroll
         for (int q = 0; q < RNS_COMB; ++q) {
           const longlong2 t = *reinterpret_cast<const longlong2*>(p.odd + q * p.stride + i);
-          x.x += __mul64hi(t.x << 4, p.coef[q]);  // 2^-62 2^-60 2^64
-          x.y += __mul64hi(t.y << 4, p.coef[q]);
-          any.x |= t.x;
-          any.y |= t.y;
+          add_product(t.x, p.coef[q], hx, mx);
+          add_product(t.y, p.coef[q], hy, my);
         }
-        x.x += any.x ? RNS_COMB / 2 : 0;
-        x.y += any.y ? RNS_COMB / 2 : 0;
+        x.x += (hx << 6) + ((mx + (1ll << 25)) >> 26);
+        x.y += (hy << 6) + ((my + (1ll << 25)) >> 26);
       }
       v[r][c] = x.x;
       v[r][c + 1] = x.y;

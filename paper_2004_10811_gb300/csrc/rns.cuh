@@ -78,7 +78,7 @@ struct RnsCheb {
   const long long* sub;        // subtracted (may be C), null: none
   const long long* odd;        // RNS_COMB matrices, stride entries apart, null: none ...
   int64_t stride;
-  long long coef[RNS_COMB];    // ... combined with these 2^-60 coefficients, and added
+  long long coef[RNS_COMB];    // ... combined with these 2^-58 coefficients, and added
   long long* C;                // the result (upper tiles), null: not stored
   __nv_bfloat16* R;            // its residues (both triangles), null: none
   double* out;                 // out_scale times the result, complete FP64 (may be C's memory), null: none
