@@ -48,7 +48,7 @@ FP64_NOMINAL_GFLOPS = 1250.0   # GB300 FP64 rate (recipe's nominal table)
 FP32_NOMINAL_GFLOPS = 152 * 128 * 2 * 2.07
 L2_BYTES = 129 << 20           # GB300 L2
 CLASS_NAMES = ["tc_gemm_newton_schulz", "tc_gemm_correction", "simt_gemm_fp64", "gather",
-               "tc_gemm_sliced_fp64", "tc_gemm_adjoint", "scatter", "reserved"]
+               "tc_gemm_sliced_fp64", "tc_gemm_adjoint", "scatter", "residue_products_fp64"]
 NCLASS = len(CLASS_NAMES)
 HBM_CLASSES = (3, 6)   # byte-counted kernels: gather, scatter
 
@@ -744,7 +744,7 @@ def main():
                 cls = 2
                 adj_prec = "fp64" if args.prec == "fp64" else "fp32"
                 peak = FP64_NOMINAL_GFLOPS / 1e3 if adj_prec == "fp64" else FP32_NOMINAL_GFLOPS / 1e3
-                roof = {"kernel": "k_gemm_simt", "bound": "alu", "peak": peak,
+                roof = {"kernel": f"k_gemm_f{64 if adj_prec == 'fp64' else 32}", "bound": "alu", "peak": peak,
                         "peak_source": "nominal FP64" if adj_prec == "fp64" else
                         "nominal FP32 (152 SMs x 128 lanes x 2 x 2.07 GHz)"}
             else:

@@ -124,8 +124,9 @@ typedef struct {
                                   that evaluates D returns D = f(K - mu I),
                                   f(x) = 1 / (1 + exp(x / kT)) = (1 - tanh(x / 2kT)) / 2, per
                                   submatrix by a Chebyshev series of tanh (truncation below
-                                  1e-13 for FP64 plans, 1e-8 for FP32) on the SIMT GEMM in the
-                                  plan's precision; mixed plans return UNSUPPORTED.  The
+                                  1e-13 for FP64 plans, 1e-8 for FP32) on FP64-accurate residue
+                                  products (FP64) or the FP32 SIMT GEMM; mixed plans return
+                                  UNSUPPORTED.  The
                                   series degree grows like (spectral scale) / kT: a degree
                                   above 8191 returns UNSUPPORTED.  submat_mu_search then takes
                                   Newton steps on the smooth Tr D(mu) (submat_stats.dn_dmu),
@@ -354,7 +355,7 @@ submat_status submat_get_sub_stats(const submat_plan* plan, int32_t* dims, int32
  *
  *   D = 1/2 (I - sign(K - mu I))  for one dense symmetric n x n matrix K,
  *
- * by scaled FP64 Newton-Schulz iteration on the FP64 path's kernels, with
+ * by scaled FP64 Newton-Schulz iteration in one cooperative launch, with
  * X_0 = (K - mu I) / beta and beta = min(max row abs-sum, ||K - mu I||_F),
  * the rigorous bound only (no power-estimate tightening, so it may take a
  * few more iterations than a plan), for callers that may not call
@@ -376,7 +377,8 @@ submat_status submat_get_sub_stats(const submat_plan* plan, int32_t* dims, int32
  * array and it keeps the previous call's contents, so calls whose work
  * overlaps on the GPU (other streams, other host threads) race; serialise
  * them.  The call synchronises `stream`.
- * Returns OK, INVALID_ARG, NONFINITE, NOT_CONVERGED (D written), CUDA.
+ * Returns OK, INVALID_ARG, NONFINITE, NOT_CONVERGED (D written), TIMEOUT (a
+ * grid barrier waited 2 s), CUDA.
  */
 #define SUBMAT_NOALLOC_MAX_N 512
 submat_status submat_dense_sign_noalloc(int n, const double* K_dev, double mu, double* D_dev,

@@ -161,7 +161,8 @@ namespace {
 // sums[k] = sum_n g_n cos(k theta_n), one thread per k in ascending n, as the host
 // does.  The N^2 / 2 terms took the host 10 ms an evaluation at degree ~400 (N =
 // 2048), a third of it; here a chain of N multiply-adds per warp, spread over the
-// SMs, takes ~0.1 ms: FP32 mu search 171.3 -> 120.4 ms, FP64 build 28.3 -> 26.4.
+// SMs, takes ~0.1 ms: FP32 mu search 171.3 -> 120.4 ms, FP64 build
+// of 240 submatrices 28.3 -> 26.4.
 __global__ void __launch_bounds__(32) k_cheb_sums(int N, int ncoef, const double* __restrict__ g,
                                                   const double* __restrict__ cosv, double* __restrict__ sums) {
   const int k = blockIdx.x * 32 + threadIdx.x;
@@ -497,7 +498,7 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
 // and T_2 in FP64.  Every T_k has norm 1 or less; the Clenshaw terms move as
 // b_j 2^-e (fermi_clenshaw_exponent).  Residue set 0 holds the factor that
 // stays (T_2, then Y), set 1 the one that each pass renews.
-// 720 submatrices of 240 molecules (13 + 5 + 5 functions, 6.5 A, kT 0.05): a
+// 240 submatrices of 219-384 dims (blocks of 13, 5 and 5 functions, kT 0.05): a
 // build took 573 ms with the FP64 SIMT GEMM and takes 24.9 ms, 10.5 of them in
 // the giant steps' passes (k_rns_cheb).
 submat_status Plan::fermi_rns(int wi, const FermiPoly& P, double** out, int* products, cudaStream_t st) {

@@ -259,7 +259,8 @@ struct Plan {
   submat_status sign_fermi(const double* K, double mu, double* D, cudaStream_t st);
   // one wave of the finite-temperature evaluation on workspace `w` of E
   // elements per buffer, wi its index for residue products (-1: SIMT); with
-  // Dbar set, the polynomial runs on dual numbers and -1/2 of its derivative part (L_f(a_j, G_j)) is added into Kbar
+  // Dbar set, the polynomial runs on dual numbers and -1/2 of its derivative
+  // part (L_f(a_j, G_j)) is added into Kbar
   template <typename T>
   submat_status fermi_wave(Wave& wv, int wi, const double* K, double mu, double* D, const double* Dbar, double* Kbar,
                            void* w, int64_t E, cudaStream_t st);
