@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <functional>
+#include <limits>
 
 #include "plan.cuh"
 
@@ -78,11 +79,13 @@ submat_status mu_bisect(const std::function<submat_status(double, double*)>& eva
   double far = up ? hi : lo;  // not evaluated
   double best_mu = side0 == 0 ? mu0 : HUGE_VAL, best_n = n0;
   double width_floor = 1e-10 * std::max(bmax, 1e-300);
+  // evaluations on one plateau differ by the rounding of the trace
+  const double rounding = 8.0 * std::numeric_limits<double>::epsilon() * std::max(1.0, std::fabs(n_el));
   auto consider = [&](double mu, double nm) {
     last_mu = mu;
     // the latest of the evaluations nearest n_el: at a step of the staircase
     // that is an end of the final bracket
-    if (std::fabs(nm - n_el) <= std::fabs(best_n - n_el)) { best_mu = mu; best_n = nm; }
+    if (std::fabs(nm - n_el) <= std::fabs(best_n - n_el) + rounding) { best_mu = mu; best_n = nm; }
   };
   bool far_ok = false;  // N(far) has been seen on the other side of n_el
   while (r.steps + r.probes < max_steps && (hi - lo) > width_floor) {
