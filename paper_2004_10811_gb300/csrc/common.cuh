@@ -257,6 +257,49 @@ __device__ __forceinline__ float d2f_trunc(double x) {
   return __uint_as_float((sign << 31) | (unsigned(ex + 127) << 23) | mant);
 }
 
+// s + e = a + b exactly (intrinsics, so that nothing is contracted)
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  const float t = __fadd_rn(a, b), v = __fsub_rn(t, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, v)), __fsub_rn(b, v));
+  s = t;
+}
+
+// A running sum in three FP32 parts, for sums that have to keep FP64's accuracy
+// where its pipe (a warp's instruction holds it for 64 clocks) would be the bound:
+// parts of 24 bits each, so more than FP64's 53 over any number of terms.
+struct Sum3 {
+  float h = 0.0f, m = 0.0f, l = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    float e;
+    two_sum(h, x, h, e);
+    two_sum(m, e, m, e);
+    l = __fadd_rn(l, e);
+  }
+  // weight (a + b)^2, weight a power of two and b at most half a unit of a
+  __device__ __forceinline__ void add_square(float a, float b, float weight) {
+    const float p = __fmul_rn(a, a);
+    float e = __fmaf_rn(2.0f * a, b, __fmaf_rn(a, a, -p));
+    add(weight * p);
+    two_sum(m, weight * e, m, e);
+    l = __fadd_rn(l, e);
+  }
+  __device__ __forceinline__ double value() const { return double(h) + (double(m) + double(l)); }
+};
+
+// adds the block's sum of part into *out (WARPS warps)
+template <int WARPS>
+__device__ __forceinline__ void add_block_sum(double part, double* out) {
+  __shared__ double red[WARPS];
+  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int q = 0; q < WARPS; ++q) t += red[q];
+    if (t != 0.0) atomicAdd(out, t);
+  }
+}
+
 // FP32 -> FP64 exactly, with integer operations
 __device__ __forceinline__ double f2d_exact(float f) {
   const unsigned u = __float_as_uint(f);

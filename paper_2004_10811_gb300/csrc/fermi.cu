@@ -215,15 +215,16 @@ __global__ void k_fermi_scale_sq(WaveDev w, T* __restrict__ M, const double* __r
 
 // W = sum_i r_i T_{2i+1} - B (B may be null): the giant-step coefficient R_j
 // less the Clenshaw term b_{j+2}.  W may be B (each entry is read, then
-// written by the same thread).
+// written by the same thread).  With route, only the submatrices of the chains.
 struct CombArgs {
   double r[kFermiBaby / 2];
 };
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_cheb_comb(WaveDev w, const T* __restrict__ odd, int64_t stride,
-                                                   CombArgs ca, const T* B, T* W) {
+                                                   CombArgs ca, const T* B, T* W, const int* __restrict__ route) {
   const int s = blockIdx.y;
+  if (route && route[s] == ST_ACTIVE) return;
   const int ld = w.ld[s];
   const int64_t total = int64_t(ld) * ld, base = w.off[s];
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
@@ -242,10 +243,11 @@ __global__ void __launch_bounds__(256) k_cheb_comb(WaveDev w, const T* __restric
 template <typename T>
 __global__ void __launch_bounds__(256) k_cheb_comb_upper(WaveDev w, const int4* __restrict__ items,
                                                          const T* __restrict__ odd, int64_t stride, CombArgs ca,
-                                                         const T* B, T* W) {
+                                                         const T* B, T* W, const int* __restrict__ route) {
   constexpr int V = 16 / sizeof(T);  // entries of a 16-byte access
   struct alignas(16) Vec { T v[V]; };
   const int4 item = items[blockIdx.x];
+  if (route && route[item.x] == ST_ACTIVE) return;
   const int ld = w.ld[item.x];
   const int64_t base = w.off[item.x] + int64_t(item.y) * 64 * ld + item.z * 64;
   for (int e = threadIdx.x; e < 64 * 64 / V; e += 256) {
@@ -355,6 +357,8 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
     SM_TRY(timer.stop(tk, st));
     return SUBMAT_OK;
   };
+  // submatrices of the FP64 chains on a wave of residue products (null: all)
+  const int* route = nullptr;
   // C = alpha A B + beta C0 + diag I (symmetric: A, B commute), and with
   // dual numbers C' = alpha (A' B + A B') + beta C0' (full tiles)
   auto gemm = [&](const T* Aop, const T* Bop, const T* C0, T* C, double alpha, double beta,
@@ -363,7 +367,7 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
     a.w = wv.dev; a.items = wv.sym64; a.nitems = wv.n_sym64;
     a.A = Aop; a.B = Bop; a.C0 = C0; a.C = C;
     a.alpha = alpha; a.beta = beta; a.diag = diag; a.sym = 1;
-    a.res2 = nullptr; a.state = nullptr; a.skip_state = -1;
+    a.res2 = nullptr; a.state = route; a.skip_state = ST_ACTIVE;
     if (dual) {  // derivative first: it reads the values of A, B (and C0 may alias C)
       Args d = a;
       d.items = wv.full64; d.nitems = wv.n_full64; d.sym = 0; d.diag = 0.0;
@@ -379,8 +383,8 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
   // T_2 = 2 X^2 - I at X = a / beta_bound, and from it the tight scale
   const bool residues = wi >= 0;  // FP64 forward only
   if (residues) {
-    long long* F = reinterpret_cast<long long*>(A);  // A has served its purpose
-    SM_CUDA(launch_rns_convert(wv.dev, reinterpret_cast<double*>(odd), nullptr, nullptr, 0, rns_residues(1), nullptr,
+    const RnsSum F = fermi_rns_sum();  // in A's memory, which has served its purpose
+    SM_CUDA(launch_rns_convert(wv.dev, reinterpret_cast<double*>(odd), nullptr, nullptr, 0, rns_residues(1), RnsFix{},
                                max_ld(wv), st));
     SM_TRY(rns_product(size_t(wi), 1, 1, F, nullptr, st));
     SM_CUDA(launch_rns_cheb2(wv.dev, F, reinterpret_cast<double*>(T2), max_ld(wv), st));
@@ -426,19 +430,21 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
     k_fermi_scale_sq<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, dp(T2), ns.cscale);
     SM_KCHECK();
   }
-  FermiPoly P;
+  if (residues) SM_TRY(rns_route(size_t(wi), reinterpret_cast<const double*>(odd), nullptr, &route, st));
+  FermiPoly P;  // its transform waits for the stream
   SM_TRY(fermi_poly(sigma / (2.0 * opt.kT), tol_poly, kFermiMaxDegree, &P,
                     [&](const std::vector<double>& g, const std::vector<double>& cosv, int ncoef, double* sums) {
                       return cheb_transform(g, cosv, ncoef, sums, st);
                     }));
   fermi_degree = std::max(fermi_degree, P.m);
   fermi_trunc = std::max(fermi_trunc, P.trunc);
-  T* out = nullptr;
-  if (residues) {
-    double* o = nullptr;
-    SM_TRY(fermi_rns(wi, P, &o, &products, st));
-    out = reinterpret_cast<T*>(o);
-  } else {
+  T* out = bb[0];
+  const bool chains = residues && static_cast<const int*>(h_pinned)[1] > 0;
+  if (residues) SM_TRY(fermi_rns(wi, P, route, &products, st));
+  if (chains) SM_TRY(collect_route(wv, st));
+  if (!residues || chains) {
+    const int counted = products;
+    if (chains) SM_TRY(gemm(odd, odd, nullptr, T2, 2.0, 0.0, -1.0));
     // baby steps: T_3 = 2 T_2 X - X, T_{k+2} = 2 T_2 T_k - T_{k-2}
     for (int q = 1; q < S / 2; ++q)
       SM_TRY(gemm(T2, odd + int64_t(q - 1) * E, q >= 2 ? odd + int64_t(q - 2) * E : odd, odd + int64_t(q) * E,
@@ -450,32 +456,24 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
     auto comb = [&](int j, const T* B, T* W, bool upper) -> submat_status {
       CombArgs ca;
       for (int q = 0; q < S / 2; ++q) ca.r[q] = P.r[size_t(j) * (S / 2) + q];
-      if (upper) k_cheb_comb_upper<T><<<wv.n_sym64, 256, 0, st>>>(wv.dev, wv.sym64, odd, E, ca, B, W);
-      else k_cheb_comb<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, odd, E, ca, B, W);
+      if (upper) k_cheb_comb_upper<T><<<wv.n_sym64, 256, 0, st>>>(wv.dev, wv.sym64, odd, E, ca, B, W, route);
+      else k_cheb_comb<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, odd, E, ca, B, W, route);
       SM_KCHECK();
       if (dual) {
-        k_cheb_comb<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, dp(odd), E, ca, dp(B), dp(W));
+        k_cheb_comb<T><<<fermi_grid(wv), 256, 0, st>>>(wv.dev, dp(odd), E, ca, dp(B), dp(W), nullptr);
         SM_KCHECK();
       }
       return SUBMAT_OK;
     };
-    if (P.blocks == 1) {
-      SM_TRY(comb(0, nullptr, bb[0], false));
-      out = bb[0];
-    } else {
-      T* b1 = bb[0];     // b_{j+1}
-      T* b2 = nullptr;   // b_{j+2} (b_G = 0 at the start)
-      SM_TRY(comb(P.blocks - 1, nullptr, b1, false));
-      for (int j = P.blocks - 2; j >= 0; --j) {
-        // W = R_j - b_{j+2} (in place over b_{j+2}), then W += c Y b_{j+1}
-        T* W = b2 ? b2 : bb[1];
-        SM_TRY(comb(j, b2, W, true));  // W is the product's C0
-        SM_TRY(gemm(Y, b1, W, W, j == 0 ? 1.0 : 2.0, 1.0, 0.0));
-        if (j == 0) { out = W; break; }
-        b2 = b1;
-        b1 = W;
-      }
+    // b_j in bb[j mod 2], over b_{j+2}
+    SM_TRY(comb(P.blocks - 1, nullptr, bb[(P.blocks - 1) & 1], false));
+    for (int j = P.blocks - 2; j >= 0; --j) {
+      // W = R_j - b_{j+2} (in place), then W += c Y b_{j+1}
+      T* W = bb[j & 1];
+      SM_TRY(comb(j, j < P.blocks - 2 ? W : nullptr, W, true));  // W is the product's C0
+      SM_TRY(gemm(Y, bb[(j + 1) & 1], W, W, j == 0 ? 1.0 : 2.0, 1.0, 0.0));
     }
+    if (chains) products = counted;  // the same products, on the other submatrices
   }
   SM_CUDA(cudaEventRecord(ev[2], st));
   // D = (I - p(X)) / 2 on the extracted columns, Tr and sum of squares
@@ -494,45 +492,55 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
   return SUBMAT_OK;
 }
 
+RnsSum Plan::fermi_rns_sum() const {
+  double* w = static_cast<double*>(ws);
+  return RnsSum{reinterpret_cast<long long*>(w), reinterpret_cast<int*>(w + (1 + kFermiBuffers) * ws_elems)};
+}
+
 // The recurrences of fermi_wave on exact residue products (rns.cuh), from X
-// and T_2 in FP64.  Every T_k has norm 1 or less; the Clenshaw terms move as
-// b_j 2^-e (fermi_clenshaw_exponent).  Residue set 0 holds the factor that
+// and T_2 in FP64, to p(X) in FP64 in the first Clenshaw buffer; submatrices of the
+// chains are left as they are.  Every T_k has norm 1 or less; the Clenshaw terms
+// move as b_j 2^-e (fermi_clenshaw_exponent).  Residue set 0 holds the factor that
 // stays (T_2, then Y), set 1 the one that each pass renews.
 // 240 submatrices of 219-384 dims (blocks of 13, 5 and 5 functions, kT 0.05): a
-// build took 573 ms with the FP64 SIMT GEMM and takes 24.9 ms, 10.5 of them in
-// the giant steps' passes (k_rns_cheb).
-submat_status Plan::fermi_rns(int wi, const FermiPoly& P, double** out, int* products, cudaStream_t st) {
+// build takes 33.6 ms, 15.4 of them in the products, against 574 ms with the FP64
+// SIMT GEMM.
+submat_status Plan::fermi_rns(int wi, const FermiPoly& P, const int* route, int* products, cudaStream_t st) {
   constexpr int H = kFermiBaby / 2;
   static_assert(H == RNS_COMB, "one coefficient per stored odd T_k");
   const Wave& wv = waves[size_t(wi)];
   const int64_t E = ws_elems;
   const int mld = max_ld(wv), e = fermi_clenshaw_exponent(P);
-  long long* F = static_cast<long long*>(ws);
-  long long* odd = F + E;
-  long long* T2 = odd + H * E;
-  long long* bb[2] = {T2 + E, T2 + 2 * E};
+  const RnsSum F = fermi_rns_sum();
+  auto fix = [&](int k) {  // the k-th FP64 buffer of fermi_wave: the odd T_k, T_2 / Y, two Clenshaw terms
+    return RnsFix{F.f + (1 + k) * E, reinterpret_cast<unsigned short*>(F.g + E) + k * E};
+  };
+  auto odd = [&](int q) { return fix(q); };
+  const RnsFix T2 = fix(H);
   __nv_bfloat16* R[2] = {rns_residues(0), rns_residues(1)};
   auto product = [&]() -> submat_status {  // F = (set 0) (set 1)
     ++*products;
-    return rns_product(size_t(wi), 0, 1, F, nullptr, st);
+    return rns_product(size_t(wi), 0, 1, F, route, st);
   };
-  auto dbl = [](long long* p) { return reinterpret_cast<double*>(p); };
-  SM_CUDA(launch_rns_convert(wv.dev, dbl(odd), nullptr, nullptr, 0, R[1], odd, mld, st));
-  SM_CUDA(launch_rns_convert(wv.dev, dbl(T2), nullptr, nullptr, 0, R[0], T2, mld, st));
+  auto dbl = [](const RnsFix& x) { return reinterpret_cast<double*>(x.hi); };
+  SM_CUDA(launch_rns_convert(wv.dev, dbl(odd(0)), route, nullptr, 0, R[1], odd(0), mld, st));
+  SM_CUDA(launch_rns_convert(wv.dev, dbl(T2), route, nullptr, 0, R[0], T2, mld, st));
   RnsCheb c{};
+  c.state = route;
   c.F = F;
   c.twice = 1;
   c.R = R[1];
   for (int q = 1; q < H; ++q) {  // T_{2q+1} = 2 T_2 T_{2q-1} - T_{2q-3}, T_{-1} = T_1
     SM_TRY(product());
-    c.sub = odd + int64_t(std::max(0, q - 2)) * E;
-    c.C = odd + int64_t(q) * E;
+    c.sub = odd(std::max(0, q - 2));
+    c.C = odd(q);
     if (q == H - 1) c.R = nullptr;
     SM_CUDA(launch_rns_cheb(wv.dev, c, mld, st));
   }
   for (int i = 0; i < 2; ++i) {  // residues of -T_9 and -T_7
     RnsCheb t{};
-    t.sub = odd + int64_t(H / 2 - i) * E;
+    t.state = route;
+    t.sub = odd(H / 2 - i);
     t.R = R[i];
     SM_CUDA(launch_rns_cheb(wv.dev, t, mld, st));
   }
@@ -543,25 +551,25 @@ submat_status Plan::fermi_rns(int wi, const FermiPoly& P, double** out, int* pro
   SM_CUDA(launch_rns_cheb(wv.dev, c, mld, st));
   // giant steps: b_j = R_j + 2 Y b_{j+1} - b_{j+2}, p = R_0 + Y b_1 - b_2
   c = RnsCheb{};
-  c.odd = odd;
+  c.state = route;
+  c.odd = odd(0);
   c.stride = E;
   c.R = R[1];
   for (int j = P.blocks - 1; j >= 0; --j) {
-    long long* W = bb[j & 1];  // b_{j+2}'s place
-    for (int q = 0; q < H; ++q) c.coef[q] = std::llrint(std::ldexp(P.r[size_t(j) * H + q], RNS_FRAC - e));
+    const RnsFix W = fix(H + 1 + (j & 1));  // b_{j+2}'s place
+    for (int q = 0; q < H; ++q) c.coef[q] = std::llrint(std::ldexp(P.r[size_t(j) * H + q], RNS_COEF - e));
     if (j < P.blocks - 1) {
       SM_TRY(product());
       c.F = F;
     }
     c.twice = j > 0;
-    c.sub = j < P.blocks - 2 ? W : nullptr;
+    c.sub = j < P.blocks - 2 ? W : RnsFix{};
     c.C = W;
     if (j == 0) {
-      c.C = nullptr;
+      c.C = RnsFix{};
       c.R = nullptr;
       c.out = dbl(W);
-      c.out_scale = std::ldexp(1.0, e - RNS_FRAC);
-      *out = c.out;
+      c.out_scale = std::ldexp(1.0, e);
     }
     SM_CUDA(launch_rns_cheb(wv.dev, c, mld, st));
   }

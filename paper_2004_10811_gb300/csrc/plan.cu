@@ -463,15 +463,16 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
   SM_CUDA(cudaMemGetInfo(&fre, &tot));
   if (cap == 0) cap = size_t(double(fre) * 0.8);
   if (opt.prec == SUBMAT_FP64) {
-    // residue products (72 B per element, 152 B at finite temperature) wherever
-    // the largest submatrix fits the workspace that way (21x faster at 420-480
-    // dims, and never slower: one 64-wide SIMT tile alone takes ~65 us); the
-    // SIMT GEMM (24 B and 96 B) below that
+    // residue products (98 B per element, 198 B at finite temperature; 72 B with
+    // the moduli in two parts) wherever the largest submatrix fits the workspace
+    // that way; the SIMT GEMM (24 B and 96 B) below that
     const size_t ld = size_t(n_max + 63) / 64 * 64;
     const size_t room = std::min(cap, size_t(double(fre) * 0.8));
-    use_rns = ld * ld * (rns_state_bytes() + rns_residue_bytes()) <= room;
+    for (rns_parts = 1; rns_parts <= (opt.kT > 0.0 ? 1 : 2) && !use_rns; ++rns_parts)
+      use_rns = ld * ld * rns_bytes() <= room && rns_route_fits(int(ld));
+    --rns_parts;
     if (use_rns) {
-      bpe = rns_state_bytes() + rns_residue_bytes();
+      bpe = rns_bytes();
       cap = room;
     }
   }
@@ -527,6 +528,7 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
   res_beta.assign(nq, 0.0);
   res_bound.assign(nq, 0.0);
   res_notconv.assign(nq, 0);
+  res_chain.assign(nq, 0);
   SM_CUDA(cudaStreamSynchronize(st));
   return SUBMAT_OK;
 }
@@ -664,31 +666,40 @@ submat_status Plan::ns_simt(const Wave& wv, T* buf0, T* buf1, T* Y, double tol, 
 struct RnsState {
   std::vector<CUtensorMap*> maps;  // per wave: [residue set][bucket]
   unsigned* norm2 = nullptr;       // per slot
+  unsigned* least = nullptr;       // per slot: coupling measure of launch_rns_route
+  int* route = nullptr;            // per slot: ST_DONE for the FP64 chains
 };
 
 void free_rns(void* state) { delete static_cast<RnsState*>(state); }
 
 // Bytes per dense element: the matrices that precede the residue sets in the
-// workspace (X and F, or the buffers of fermi_wave), and the two sets.
-size_t Plan::rns_state_bytes() const { return opt.kT > 0.0 ? fermi_bytes_per_elem(SUBMAT_FP64) : 16; }
-size_t rns_residue_bytes() { return 2 * 2 * RNS_MODS; }
+// workspace, and the two sets.  T = 0: X.hi, F.f and F.g, X.lo, and with the moduli
+// in two parts Y.hi, Y.lo; T > 0: the FP64 buffers of fermi_wave (A's memory is
+// F.f, the others are hi parts), F.g, and the lo parts.  The buffers of the SIMT
+// GEMM start at the same place.
+size_t Plan::rns_state_bytes() const {
+  if (opt.kT > 0.0) return fermi_bytes_per_elem(SUBMAT_FP64) + 4 + 2 * kFermiBuffers;
+  return 8 + 8 + 4 + 2 + (rns_parts == 2 ? 10 : 0);
+}
+size_t Plan::rns_bytes() const { return rns_state_bytes() + 2 * 2 * rns_planes(rns_parts); }
 
 __nv_bfloat16* Plan::rns_residues(int set) const {
   return reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(ws) + rns_state_bytes() * size_t(ws_elems)) +
-         int64_t(set) * RNS_MODS * ws_elems;
+         int64_t(set) * rns_planes(rns_parts) * ws_elems;
 }
 
 // Tensor maps of the two residue sets.
 submat_status Plan::rns_setup(cudaStream_t st) {
   std::unique_ptr<RnsState> r(new RnsState());
   __nv_bfloat16* base = rns_residues(0);
+  const int planes = rns_planes(rns_parts);
   for (auto& wv : waves) {
     const size_t nbk = wv.bucket_ld.size();
     std::vector<CUtensorMap> maps(2 * nbk);
     for (size_t i = 0; i < 2 * nbk; ++i) {
       const size_t k = i % nbk;
-      const __nv_bfloat16* p = base + RNS_MODS * (int64_t(i / nbk) * ws_elems + wv.bucket_base[k]);
-      if (make_bucket_map(&maps[i], p, int(wv.bucket_ld[k]), wv.bucket_count[k] * RNS_MODS) != 0) {
+      const __nv_bfloat16* p = base + planes * (int64_t(i / nbk) * ws_elems + wv.bucket_base[k]);
+      if (make_bucket_map(&maps[i], p, int(wv.bucket_ld[k]), wv.bucket_count[k] * planes) != 0) {
         set_error("cuTensorMapEncodeTiled failed");
         return SUBMAT_ERR_CUDA;
       }
@@ -698,14 +709,19 @@ submat_status Plan::rns_setup(cudaStream_t st) {
     SM_CUDA(cudaStreamSynchronize(st));  // the host array goes out of scope
     r->maps.push_back(d);
   }
-  SM_TRY(alloc(&r->norm2, size_t(max_wave), "row norms"));
+  int slots = 0;
+  for (auto& wv : waves) slots = std::max(slots, wv.count);
+  SM_TRY(alloc(&r->norm2, size_t(slots), "row norms"));
+  SM_TRY(alloc(&r->least, size_t(slots), "coupling measures"));
+  SM_TRY(alloc(&r->route, size_t(slots), "routes"));
   rns = r.release();
   return SUBMAT_OK;
 }
 
 // F = frac of the symmetric product of two residue sets on the upper tiles of a
-// wave; submatrices with state ST_DONE are skipped.
-submat_status Plan::rns_product(size_t wi, int a, int b, long long* F, const int* state, cudaStream_t st) {
+// wave (its sums over one part of the moduli, added to those of an earlier one);
+// submatrices with state ST_DONE are skipped.
+submat_status Plan::rns_product(size_t wi, int a, int b, RnsSum F, const int* state, cudaStream_t st, int part) {
   const Wave& wv = waves[wi];
   const size_t nbk = wv.bucket_ld.size();
   const int nsm = num_sms();
@@ -716,11 +732,18 @@ submat_status Plan::rns_product(size_t wi, int a, int b, long long* F, const int
   p.map_b = maps + size_t(b) * nbk;
   p.off = wv.dev.off; p.ld = wv.dev.ld;
   p.state = state; p.skip_state = ST_DONE;
-  p.split = rns_split(p.nitems, nsm);
+  p.planes = rns_planes(rns_parts);
+  p.mod0 = part * p.planes;
+  p.nmod = std::min(p.planes, RNS_MODS - p.mod0);
+  p.add = part > 0;
+  p.split = rns_split(p.nitems, p.nmod, nsm);
   p.F = F;
   p.flags = d_flags;
   p.timeout_cycles = kWaitCycles;
-  if (p.split > 1) SM_CUDA(cudaMemsetAsync(F, 0, size_t(wv.elems) * 8, st));
+  if (p.split > 1 && !p.add) {
+    SM_CUDA(cudaMemsetAsync(F.f, 0, size_t(wv.elems) * 8, st));
+    SM_CUDA(cudaMemsetAsync(F.g, 0, size_t(wv.elems) * 4, st));
+  }
   size_t tk;
   SM_TRY(timer.start(KC_RNS, st, &tk));
   SM_CUDA(launch_rns_gemm(p, nsm, st));
@@ -728,54 +751,114 @@ submat_status Plan::rns_product(size_t wi, int a, int b, long long* F, const int
   return SUBMAT_OK;
 }
 
+// Decides which of a wave's submatrices the FP64 chains evaluate (rns.cuh); their
+// number is in h_pinned[1] once the stream has been waited for.
+submat_status Plan::rns_route(size_t wi, const double* X, int* state, const int** route, cudaStream_t st) {
+  const Wave& wv = waves[wi];
+  auto* r = static_cast<RnsState*>(rns);
+  SM_CUDA(launch_rns_route(g, wv.dev, X, state, r->least, r->route, d_active, nb_max, max_ld(wv), st));
+  SM_CUDA(cudaMemcpyAsync(static_cast<int*>(h_pinned) + 1, d_active, sizeof(int), cudaMemcpyDeviceToHost, st));
+  if (route) *route = r->route;
+  return SUBMAT_OK;
+}
+
+// Per-submatrix routes of a wave with chains, for the statistics.
+submat_status Plan::collect_route(const Wave& wv, cudaStream_t st) {
+  std::vector<int> rt(wv.count);
+  SM_CUDA(cudaMemcpyAsync(rt.data(), static_cast<const RnsState*>(rns)->route, sizeof(int) * wv.count,
+                          cudaMemcpyDeviceToHost, st));
+  SM_CUDA(cudaStreamSynchronize(st));
+  for (int s = 0; s < wv.count; ++s) res_chain[wv.first + s] = rt[s] == ST_DONE;
+  return SUBMAT_OK;
+}
+
 // Newton-Schulz on one wave with X_0 = a / beta in the first buffer, which ends
-// as sign(a).  X moves as 2^-58 fixed point on its upper tiles; a product pass
+// as sign(a) (ns.par 0; submatrices of the chains: as ns_simt leaves them).  X
+// moves in fixed point on its upper tiles; a product pass
 // (F on upper 128 x 128 tiles) and a pass over 64 x 64 tile pairs alternate.
 // The first square keeps FP64 and measured operand scales, since rho(X_0) is
 // certified only from it; from then on rho(X) and rho(X^2) are at most 1
-// (1.7146 and 2.94 for X_0, hence its shifts 1 and 2).
+// (1.7146 and 2.94 for X_0, hence its shifts 1 and 2).  With the moduli in two
+// parts, a product takes its operands' residues part by part instead of finding
+// them written by the pass before.
 submat_status Plan::ns_rns(size_t wi, cudaStream_t st) {
   const Wave& wv = waves[wi];
   auto* r = static_cast<RnsState*>(rns);
+  const bool whole = rns_parts == 1;
   double* X = static_cast<double*>(ws);
-  long long* F = reinterpret_cast<long long*>(X + ws_elems);
+  RnsSum F;
+  F.f = reinterpret_cast<long long*>(X + ws_elems);
+  F.g = reinterpret_cast<int*>(F.f + ws_elems);
+  unsigned short* lo = reinterpret_cast<unsigned short*>(F.g + ws_elems);
+  const RnsFix fix{reinterpret_cast<long long*>(X), lo};
+  RnsFix Y{};
+  if (!whole) {
+    Y.hi = reinterpret_cast<long long*>(lo + ws_elems);
+    Y.lo = reinterpret_cast<unsigned short*>(Y.hi + ws_elems);
+  }
+  double* Y0 = reinterpret_cast<double*>(whole ? F.f : Y.hi);  // the first square
   __nv_bfloat16* R[2] = {rns_residues(0), rns_residues(1)};
   const int mld = max_ld(wv);
-  auto product = [&](int b) { return rns_product(wi, 0, b, F, ns.state, st); };  // F = X (b = 0: X, 1: Y)
+  // F = (set 0) (set b); operands(part) writes the residues that are not there yet
+  auto product = [&](int b, const std::function<submat_status(int)>& operands) -> submat_status {
+    for (int part = 0; part < rns_parts; ++part) {
+      SM_TRY(operands(part));
+      SM_TRY(rns_product(wi, 0, b, F, ns.state, st, part));
+    }
+    return SUBMAT_OK;
+  };
+  auto spread = [&](RnsFix x, int set, int part) -> submat_status {
+    if (!whole) SM_CUDA(launch_rns_spread(wv.dev, ns.state, x, R[set], mld, st, part));
+    return SUBMAT_OK;
+  };
+  SM_TRY(rns_route(wi, X, ns.state, nullptr, st));
   for (int k = 0; k < opt.max_iter; ++k) {
     if (k == 0) {
       SM_CUDA(launch_rns_rownorm(wv.dev, X, ns.state, r->norm2, mld, st));
-      SM_CUDA(launch_rns_convert(wv.dev, X, ns.state, r->norm2, 0, R[0], nullptr, mld, st));
-      SM_TRY(product(0));
-      SM_CUDA(launch_rns_square0(wv.dev, ns, r->norm2, F, mld, st));
+      SM_TRY(product(0, [&](int part) -> submat_status {
+        SM_CUDA(launch_rns_convert(wv.dev, X, ns.state, r->norm2, 0, R[0], RnsFix{}, mld, st, rns_parts, part));
+        return SUBMAT_OK;
+      }));
+      SM_CUDA(launch_rns_square0(wv.dev, ns, r->norm2, F, Y0, mld, st));
       if (opt.beta_mode == 0) {  // the power estimate's scale, proven from X_0^2 or reduced
-        const CertSquare sq{0, F, nullptr, 1.0f, 0.0f};
+        const CertSquare sq{0, Y0, nullptr, 1.0f, 0.0f};
         const CertLinear lin{1, {X, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
         SM_CUDA(launch_certify(wv.dev, ns, sq, lin, cert_limits(false), mld, d_flags + 2, st));
       }
       SM_CUDA(launch_ns_update(wv.dev, ns, tol_eff, 1e-9, opt.max_iter, d_flags, st));
-      SM_CUDA(launch_rns_convert(wv.dev, X, ns.state, nullptr, 1, R[0], reinterpret_cast<long long*>(X), mld, st));
-      SM_CUDA(launch_rns_convert(wv.dev, reinterpret_cast<double*>(F), ns.state, nullptr, 2, R[1], nullptr, mld, st));
+      SM_TRY(product(1, [&](int part) -> submat_status {
+        SM_CUDA(launch_rns_convert(wv.dev, X, ns.state, nullptr, 1, R[0], whole ? fix : RnsFix{}, mld, st, rns_parts,
+                                   part));
+        SM_CUDA(launch_rns_convert(wv.dev, Y0, ns.state, nullptr, 2, R[1], RnsFix{}, mld, st, rns_parts, part));
+        return SUBMAT_OK;
+      }));
+      if (!whole) SM_CUDA(launch_rns_convert(wv.dev, X, ns.state, nullptr, 1, nullptr, fix, mld, st));
     } else {
-      SM_TRY(product(0));
-      SM_CUDA(launch_rns_square(wv.dev, ns, F, R[1], mld, st));
+      SM_TRY(product(0, [&](int part) { return spread(fix, 0, part); }));
+      SM_CUDA(launch_rns_square(wv.dev, ns, F, Y, whole ? R[1] : nullptr, mld, st));
       SM_CUDA(launch_ns_update(wv.dev, ns, tol_eff, 1e-9, opt.max_iter, d_flags, st));
+      SM_TRY(product(1, [&](int part) -> submat_status {
+        SM_TRY(spread(fix, 0, part));
+        return spread(Y, 1, part);
+      }));
     }
-    SM_TRY(product(1));
-    SM_CUDA(launch_rns_update(wv.dev, ns, F, k == 0 ? 3 : 0, reinterpret_cast<long long*>(X), R[0], mld, st));
+    SM_CUDA(launch_rns_update(wv.dev, ns, F, k == 0 ? 3 : 0, fix, whole ? R[0] : nullptr, mld, st));
     SM_CUDA(cudaMemsetAsync(d_active, 0, sizeof(int), st));
     SM_CUDA(launch_ns_post(wv.dev, ns, 0, d_active, st));
     SM_CUDA(cudaMemcpyAsync(h_pinned, d_active, sizeof(int), cudaMemcpyDeviceToHost, st));
     SM_CUDA(cudaStreamSynchronize(st));
     if (reinterpret_cast<int*>(h_pinned)[0] == 0) break;
   }
-  return SUBMAT_OK;
+  if (static_cast<const int*>(h_pinned)[1] == 0) return SUBMAT_OK;
+  SM_TRY(collect_route(wv, st));
+  SM_CUDA(launch_rns_resume(wv.dev, r->route, ns.state, st));
+  return ns_simt<double, GemmF64Args>(wv, X, X + ws_elems, X + 2 * ws_elems, tol_eff, 1e-9, st, launch_gemm_f64,
+                                      opt.beta_mode == 0);
 }
 
 submat_status Plan::sign_fp64(const double* K, double mu, double* D, cudaStream_t st) {
   double* B0 = static_cast<double*>(ws);
-  // residue products leave the result in the first buffer
-  double* B1 = use_rns ? B0 : B0 + ws_elems;
+  double* B1 = B0 + ws_elems;
   if (use_rns && !rns) SM_TRY(rns_setup(st));
   for (size_t wi = 0; wi < waves.size(); ++wi) {
     Wave& wv = waves[wi];
@@ -873,6 +956,7 @@ void Plan::reset_stats() {
   stats.sum_n2 = s2;
   stats.sum_n3 = s3;
   stats.workspace_bytes = ws_bytes;
+  std::fill(res_chain.begin(), res_chain.end(), 0);
   launches_at_start = launch_count();
 }
 
@@ -901,12 +985,14 @@ void Plan::finish_stats(bool adjoint) {
     if (adjoint) {  // every adjoint product runs on one GEMM kind
       stats.kernel_work[opt.adjoint_mode == 1 && opt.kT == 0.0 ? KC_TC_ADJ : KC_SIMT] += flops;
     } else if (opt.kT > 0.0) {
-      stats.kernel_work[use_rns ? KC_RNS : KC_SIMT] += flops;
+      for (int j = col_lo; j < col_hi; ++j)
+        stats.kernel_work[use_rns && !res_chain[j] ? KC_RNS : KC_SIMT] +=
+            2.0 * double(qn[j]) * qn[j] * qn[j] * res_iters[j];
     } else if (opt.prec != SUBMAT_MIXED_BF16_REFINE) {
       // two products per iteration, 2 n^3 flops each at the standard count
       for (int j = col_lo; j < col_hi; ++j) {
         const double n = qn[j];
-        stats.kernel_work[use_rns ? KC_RNS : KC_SIMT] += 4.0 * n * n * n * res_iters[j];
+        stats.kernel_work[use_rns && !res_chain[j] ? KC_RNS : KC_SIMT] += 4.0 * n * n * n * res_iters[j];
       }
     }
   }

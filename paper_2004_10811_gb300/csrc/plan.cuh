@@ -26,7 +26,6 @@ constexpr int kProbeMaxIter = 40;  // Newton-Schulz cap of a mu-search probe
 void free_mixed(void* state);
 void free_adjoint_tc(void* state);
 void free_rns(void* state);
-size_t rns_residue_bytes();  // the two residue sets of the FP64 path, per dense element
 
 // Launch plan of an exact sliced product (mixed.cu).  Slices are numbered
 // 1..n; a group is one exact accumulator: np products (pr[i] = (p, q)) of one
@@ -150,6 +149,8 @@ enum KernelClass {
 
 int max_ld(const Wave& wv);
 
+struct RnsSum;
+
 struct Plan {
   ~Plan();
 
@@ -198,6 +199,7 @@ struct Plan {
   void* mixed = nullptr;       // mixed-path state (mixed.cu)
   void* rns = nullptr;         // residue-product state of the FP64 path (plan.cu); null: SIMT GEMM
   bool use_rns = false;
+  int rns_parts = 1;           // parts of the moduli that a residue set holds one at a time
   void* adj_tc = nullptr;      // tensor-core adjoint state (mixed.cu)
   // adjoint: its own waves and workspace (six dense buffers per submatrix)
   std::vector<Wave> bwaves;
@@ -216,6 +218,7 @@ struct Plan {
 
   // results of the last evaluation (per global block column)
   std::vector<int> res_iters, res_notconv;
+  std::vector<char> res_chain;  // FP64 plans with residue products: evaluated by the chains
   std::vector<double> res_resid, res_beta, res_bound;  // res_bound: min(max row abs-sum, ||a||_F)
   int last_flags = 0;              // status word of the last read_flags
   bool probe_mode = false;         // mixed path: stop after the FP16x3 iteration (mu-search probe)
@@ -280,9 +283,13 @@ struct Plan {
   submat_status grow_ns_state(int count);
   submat_status rns_setup(cudaStream_t st);
   size_t rns_state_bytes() const;
+  size_t rns_bytes() const;
   __nv_bfloat16* rns_residues(int set) const;
-  submat_status rns_product(size_t wi, int a, int b, long long* F, const int* state, cudaStream_t st);
-  submat_status fermi_rns(int wi, const FermiPoly& P, double** out, int* products, cudaStream_t st);
+  submat_status rns_product(size_t wi, int a, int b, RnsSum F, const int* state, cudaStream_t st, int part = 0);
+  submat_status rns_route(size_t wi, const double* X, int* state, const int** route, cudaStream_t st);
+  submat_status collect_route(const Wave& wv, cudaStream_t st);
+  RnsSum fermi_rns_sum() const;
+  submat_status fermi_rns(int wi, const FermiPoly& P, const int* route, int* products, cudaStream_t st);
   submat_status ns_rns(size_t wi, cudaStream_t st);
   template <typename T, typename Args>
   submat_status ns_simt(const Wave& wv, T* buf0, T* buf1, T* Y, double tol, double floor_thr,
