@@ -172,14 +172,6 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
                : "memory");
 }
 
-// hi + lo += e^2 to about 46 bits
-__device__ __forceinline__ void add_square(float e, float& hi, float& lo) {
-  const float p = e * e, pe = fmaf(e, e, -p);
-  const float s = hi + p, b = s - hi;
-  lo += ((hi - (s - b)) + (p - b)) + pe;
-  hi = s;
-}
-
 __global__ void __launch_bounds__(64, 6) k_gemm_f32(const __grid_constant__ GemmF32Args a) {
   __shared__ __align__(16) float As[2][TK][FP];  // As[.][k][m]
   __shared__ __align__(16) float Bs[2][TK][TM];  // Bs[.][k][n]
@@ -252,8 +244,8 @@ __global__ void __launch_bounds__(64, 6) k_gemm_f32(const __grid_constant__ Gemm
   float* Cb = a.C + off;
   const float* C0b = a.C0 ? a.C0 + off : nullptr;
   const float alpha = float(a.alpha), beta = float(a.beta), diag = float(a.diag);
-  float hi = 0.0f, lo = 0.0f;  // sum of squares off the diagonal
-  double part = 0.0;           // and on it
+  Sum3 rest;          // sum of squares off the diagonal
+  double part = 0.0;  // and on it
   const int c0 = tj * TM + tx * 4;
   float v[8][8];
 #pragma unroll
@@ -277,7 +269,7 @@ __global__ void __launch_bounds__(64, 6) k_gemm_f32(const __grid_constant__ Gemm
             part = fma(e, e, part);
           }
         } else if (a.res2) {
-          add_square(x, hi, lo);
+          rest.add_square(x);
         }
         v[i][4 * h + q] = x;
       }
@@ -295,7 +287,7 @@ __global__ void __launch_bounds__(64, 6) k_gemm_f32(const __grid_constant__ Gemm
     }
   }
   if (a.res2) {
-    part += double(hi) + double(lo);
+    part += rest.value();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
     if ((tid & 31) == 0) red[tid >> 5] = part;

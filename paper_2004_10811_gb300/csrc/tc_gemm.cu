@@ -230,13 +230,6 @@ __device__ __forceinline__ void store_mirror(const TcGemmParams& p, int64_t base
   }
 }
 
-// hi + lo += x, both FP32, with the rounding error kept
-__device__ __forceinline__ void add_pair(float x, float& hi, float& lo) {
-  const float s = hi + x, b = s - hi;
-  lo += (hi - (s - b)) + (x - b);
-  hi = s;
-}
-
 template <int BN, int MODE, bool F16>
 __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const __grid_constant__ TcGemmParams p) {
   constexpr int TILE_B = BN * BK * 2;  // one BN x 64 BF16 operand tile (B side)
@@ -470,7 +463,7 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const 
         } else {
           const int side = (warp - 2) >> 2;  // chunks side, side + 2, ...
           const bool has_c0 = (p.c0_f32 || p.c0_hi) && p.beta != 0.0f && !p.dot_c0;
-          float ph = 0.0f, pl = 0.0f;  // the tile's sum for res2 or dot_c0
+          Sum3 sum;  // the tile's, for res2 or dot_c0
 #pragma unroll 1
           for (int hc = side; hc < 4 * HALVES; hc += 2) {
             const int h = hc >> 2, c = hc & 3;
@@ -518,24 +511,19 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const 
                 if (p.dot_c0) pd = fmaf(v, c0[q], pd);
               }
             }
-            if (p.res2) add_pair(p.sym && !diag_sym ? 2.0f * pr : pr, ph, pl);
-            if (p.dot_c0) add_pair(2.0f * pd, ph, pl);
+            if (p.res2) sum.add(p.sym && !diag_sym ? 2.0f * pr : pr);
+            if (p.dot_c0) sum.add(2.0f * pd);
             if (diag_sym) store_range<F16>(p, idx, o, r - c * 32);
             else store_row<F16>(p, idx, o);
             if (!p.sym || (diag_sym && c < quarter)) continue;
             store_mirror<F16>(p, base, ld, cg0, item.y * BM + quarter * 32, o, lane, diag_sym && c == quarter);
           }
-          // FP64 instructions hold their pipe for 64 clocks: sums stay in FP32
-          // pairs up to one conversion per warp
+          // FP64 instructions hold their pipe for 64 clocks: sums stay in three
+          // FP32 parts up to one conversion per warp
           if (p.res2 || p.dot_c0) {
-#pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) {
-              const float xh = __shfl_xor_sync(0xffffffffu, ph, o2), xl = __shfl_xor_sync(0xffffffffu, pl, o2);
-              add_pair(xh, ph, pl);
-              pl += xl;
-            }
+            sum.add_warp();
             if (lane == 0) {
-              const double t = double(ph) + double(pl);
+              const double t = sum.value();
               if (t != 0.0) atomicAdd(p.res2 ? &p.res2[s] : &p.dot_c0[s], t);
             }
           }

@@ -183,3 +183,23 @@ def test_water_blocks(pkg, block):
                 worst[k] = max(worst[k], float(np.linalg.norm(e.astype(float)) / np.linalg.norm(want.astype(float))))
     assert worst[0] <= worst[1], worst
 
+
+
+@pytest.mark.parametrize("beta_mode", [0, 1])
+def test_residual_sums(pkg, beta_mode):
+    """||X_0^2 - I||_F / sqrt(n), summed as FP64 sums it: a product entry is off by 2^-73
+    and the rounding of X_0, n^(1/2) 2^-53, against a residual of order 1."""
+    import torch
+    m = make_water(40, 6, 5.0, (2, -1.0, -0.3), (4, 0.3, 1.0), seed=21)
+    K = torch.from_numpy(m.vals).cuda()
+    with pkg.Plan.from_bsr(m, prec="fp64", max_iter=1, beta_mode=beta_mode) as plan:
+        plan.sign(K, 0.0, allow_not_converged=True)
+        sub = plan.sub_stats()
+    iters, resid, beta = sub["iters"], sub["resid"], sub["beta"]
+    a = bsr_to_dense(m)
+    for j in (0, 13, 39):
+        rows = m.col_idx[m.row_ptr[j]:m.row_ptr[j + 1]]
+        idx = (rows[:, None] * 6 + np.arange(6)).ravel()
+        x = a[np.ix_(idx, idx)] / beta[j]
+        want = np.linalg.norm(x @ x - np.eye(len(idx))) / np.sqrt(len(idx))
+        assert iters[j] == 1 and abs(resid[j] / want - 1) <= len(idx) ** 0.5 * 2.0 ** -50
