@@ -93,7 +93,12 @@ typedef struct {
                                   safe by itself (submat_stats.scale_reduced counts them);
                                   1: beta = min(max row abs-sum, ||a||_F) >= rho(a) only */
   int symmetrize;              /* 1: return (D + D^T) / 2 on the pattern; 0: column-assembled D */
-  size_t workspace_cap_bytes;  /* device workspace cap; 0 = 80 % of free memory at plan time */
+  size_t workspace_cap_bytes;  /* device workspace cap; 0 = 80 % of free memory at plan time (20 %
+                                  for FP64 plans, or what the largest submatrix needs).  Bytes
+                                  per entry of a wave's padded submatrices: FP64 98 (72 where
+                                  that is all that fits one submatrix; 24 below that), with
+                                  kT > 0 198 (96 below that); submat_sign_backward has its own
+                                  workspace under the same cap */
   int refine_rounds;           /* mixed path: correction rounds; 0 selects 1.  With one
                                   round a submatrix is accepted when its Lyapunov solve
                                   converged (which bounds |a|/gap); with two or more the last

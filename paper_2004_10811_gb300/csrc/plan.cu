@@ -463,9 +463,15 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
   SM_CUDA(cudaMemGetInfo(&fre, &tot));
   if (cap == 0) cap = size_t(double(fre) * 0.8);
   if (opt.prec == SUBMAT_FP64) {
-    // residue products (98 B per element, 198 B at finite temperature; 72 B with
+    // Residue products (98 B per element, 198 B at finite temperature; 72 B with
     // the moduli in two parts) wherever the largest submatrix fits the workspace
-    // that way; the SIMT GEMM (24 B and 96 B) below that
+    // that way; the SIMT GEMM (24 B and 96 B) below that.  They are 15x faster
+    // where the waves fill the chip (216 submatrices of 420-480 dims in one wave:
+    // 28.8 against 425.8 ms).  A cap of a few submatrices holds four times as many
+    // of the SIMT GEMM's, and each wave costs its launches: one residue wave per
+    // submatrix takes 548 ms there (54 SIMT waves: ~560) and for 125 of 64 dims 109
+    // (32 SIMT waves: ~52).  The line stays at what fits all the same, so that a
+    // plan's cap does not change its arithmetic.
     const size_t ld = size_t(n_max + 63) / 64 * 64;
     const size_t room = std::min(cap, size_t(double(fre) * 0.8));
     for (rns_parts = 1; rns_parts <= (opt.kT > 0.0 ? 1 : 2) && !use_rns; ++rns_parts)
@@ -473,7 +479,10 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
     --rns_parts;
     if (use_rns) {
       bpe = rns_bytes();
-      cap = room;
+      // without a cap a quarter of the SIMT GEMM's share, so that a plan takes no more
+      // of the memory for its four times as many bytes (waves of that size fill the
+      // chip many times over)
+      cap = opt.workspace_cap_bytes ? room : std::max(room / 4, ld * ld * bpe);
     }
   }
   // the evaluated submatrices (a column range without groups)

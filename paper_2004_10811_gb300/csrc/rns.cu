@@ -12,6 +12,8 @@
 
 namespace submat {
 
+int num_sms();
+
 namespace {
 
 // ---------------------------------------------------------------------------
@@ -950,10 +952,13 @@ __global__ void __launch_bounds__(256) k_rns_cheb(WaveDev w, const __grid_consta
   }
 }
 
-// about four tile pairs a block
+// about four tile pairs a block, but fewer where the wave would give less than four
+// blocks per SM
 dim3 tile_grid(int max_ld, int nsub) {
-  const int T = max_ld / 64;
-  return dim3(unsigned(std::min((T * (T + 1) / 2 + 3) / 4, 512)), unsigned(nsub));
+  const int T = max_ld / 64, pairs = T * (T + 1) / 2;
+  int per = 4;
+  while (per > 1 && int64_t((pairs + per - 1) / per) * nsub < 4 * int64_t(num_sms())) per /= 2;
+  return dim3(unsigned(std::min((pairs + per - 1) / per, 512)), unsigned(nsub));
 }
 
 }  // namespace
