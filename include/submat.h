@@ -117,8 +117,11 @@ typedef struct {
                                   1: FP64 SIMT GEMM */
   int tile_n_ns;               /* tensor-core output tile width in the Newton-Schulz phase:
                                   0 = chosen per wave, or 128 / 256 */
-  int tile_n_corr;             /* the same for the correction phase (0 = 256) */
-  int tile_n_hp;               /* the same for the sliced residual products (0 = 128) */
+  int tile_n_corr;             /* the same for the correction phase (0 = per wave: 256, or 128
+                                  where that makes fewer than two tiles per SM) */
+  int tile_n_hp;               /* the same for the sliced residual products of correction rounds
+                                  after the first (0 = 128); the first round's run in one pass
+                                  of fixed width */
   int iteration;               /* sign iteration of the mixed path: 0 (default) Newton-Schulz
                                   X <- X (3I - X^2) / 2 (Section II-B); 1 the third-order
                                   X <- X (15I - 10X^2 + 3X^4) / 8 of the paper's GPU runs
@@ -126,7 +129,7 @@ typedef struct {
                                   precisions support 0 only (UNSUPPORTED at plan creation) */
   int adjoint_mode;            /* GEMMs of submat_sign_backward: 0 (default) SIMT in the plan's
                                   precision (FP32 for mixed plans); 1 BF16x3 tensor cores, mixed
-                                  plans only (UNSUPPORTED otherwise) -- about 15x faster, with
+                                  plans only (UNSUPPORTED otherwise) -- about 3x faster, with
                                   about 10x the error of mode 0 (BF16x3 carries ~16 bits) */
   double kT;                   /* electronic temperature (Section IV-F, last paragraph: the
                                   Fermi function in place of signum), in the units of K;
@@ -334,9 +337,10 @@ submat_status submat_sign_backward(submat_plan* plan, const double* K_vals, doub
  * For a mixed-precision plan, times full evaluations of D(mu) for this K with
  * CUDA events per kernel class. The candidates are 128- and 256-wide output
  * tiles for each tensor-core phase: Newton-Schulz, correction split products
- * and sliced residual products. One untimed warm-up evaluation runs first.
- * The widths are independent per phase, so the plan keeps the faster width
- * of each, and later calls of submat_sign use them.
+ * and, with refine_rounds of 2 or more, sliced residual products (one round
+ * keeps tile_n_hp, 128 if 0, and reports it). One untimed warm-up evaluation
+ * runs first. The widths are independent per phase, so the plan keeps the
+ * faster width of each, and later calls of submat_sign use them.
  *   K_vals      device double[value count]
  *   D_vals      device double[value count] (caller-owned): receives D(mu)
  *   tile_n_out  host int[3] or NULL: the chosen widths (NS, correction, sliced)

@@ -1009,7 +1009,8 @@ void Plan::finish_stats(bool adjoint) {
 
 // Tile-width autotuner: a warm-up evaluation, then one evaluation with every
 // tensor-core phase at width 128 and one at 256, timed per kernel class; each
-// phase keeps its faster width.
+// phase keeps its faster width.  The sliced products of a single correction round
+// have one width (slice_gemm.cu): there the plan's choice stands.
 submat_status Plan::autotune(const double* K, double mu, double* D, int32_t* chosen, cudaStream_t st) {
   if (!K || !D) { set_error("K_vals and D_vals must be device pointers"); return SUBMAT_ERR_INVALID_ARG; }
   if (opt.prec != SUBMAT_MIXED_BF16_REFINE) {
@@ -1024,6 +1025,7 @@ submat_status Plan::autotune(const double* K, double mu, double* D, int32_t* cho
   const int widths[2] = {128, 256};
   const int classes[3] = {KC_TC_NS, KC_TC_REF, KC_TC_HP};
   double ms[2][3] = {{0, 0, 0}, {0, 0, 0}};
+  const int hp_was = opt.tile_n_hp ? opt.tile_n_hp : 128;
   submat_status status = SUBMAT_OK;
   for (int w = 0; w < 2 && status == SUBMAT_OK; ++w) {
     opt.tile_n_ns = opt.tile_n_corr = opt.tile_n_hp = widths[w];
@@ -1033,7 +1035,7 @@ submat_status Plan::autotune(const double* K, double mu, double* D, int32_t* cho
   timer.on = timer_was_on;
   SM_TRY(status);
   const int best[3] = {ms[1][0] < ms[0][0] ? 256 : 128, ms[1][1] < ms[0][1] ? 256 : 128,
-                       ms[1][2] < ms[0][2] ? 256 : 128};
+                       opt.refine_rounds <= 1 ? hp_was : ms[1][2] < ms[0][2] ? 256 : 128};
   opt.tile_n_ns = best[0];
   opt.tile_n_corr = best[1];
   opt.tile_n_hp = best[2];
