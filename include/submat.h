@@ -179,8 +179,9 @@ typedef struct {
    * dense element written plus 8 per K value read) and the scatter (per
    * extracted entry: the iterate read, 8 or 4 bytes, the mixed path's two
    * FP32 corrections, and 8 for D written).
-   * kernel_exec: MMA flops the tensor cores executed (every slice product,
-   * tile padding included); 0 for the other classes. */
+   * kernel_exec: MMA flops the tensor cores executed (every slice product and
+   * the padding of rows to 128 and of columns to 64 included); 0 for the
+   * other classes. */
   double  kernel_ms[8];
   int32_t kernel_launches[8];
   double  kernel_work[8];

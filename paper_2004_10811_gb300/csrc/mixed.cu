@@ -862,13 +862,12 @@ __global__ void k_scale_picked(WaveDev w, const int* __restrict__ pick, const do
   FOR_SUB_ELEMS(w) X[base + e] = A[base + e] * ib;
 }
 
-// 128 x 256 tiles with a sub-tile on or above the diagonal
-int sym256_count(int t128, int t256) {
-  int c = 0;
-  for (int a = 0; a < t128; ++a)
-    for (int b = 0; b < t256; ++b)
-      if (2 * b + 1 >= a) ++c;
-  return c;
+// MMA flops that one product of k_tc_gemm runs on a submatrix: 128 rows, the sum
+// over ld, and the columns inside the matrix that the tiles of a row form, ld of
+// them, or with a symmetric result (either tile width) ld - 128 a in row a
+double executed_flops(int ld, bool sym) {
+  const double t = (ld + 127) / 128;
+  return 2.0 * 128.0 * ld * (t * ld - (sym ? 64.0 * t * (t - 1.0) : 0.0));
 }
 
 // Blocks a submatrix gets of `units` units of work: `per` units each, few and
@@ -1080,7 +1079,6 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
       NFULL = bn == 256 ? wv.n_full256 : wv.n_full128;
     };
     use_width(opt.tile_n_ns);
-    const int ns_width = bn;
     auto tc = [&](const int4* items, int nitems, int sa0, int sa1, int sb0, int sb1, int sym,
                   float alpha, float beta) {
       TcGemmParams p;
@@ -1599,18 +1597,17 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
       if (hp_sliced) stats.kernel_work[KC_TC_HP] += 4.0 * n3 * rounds;
       else stats.kernel_work[KC_SIMT] += 4.0 * n3 * rounds;
       stats.kernel_work[KC_SIMT] += 4.0 * n3 * extra;
-      // executed MMA work: tiles x 2 * 128 * width * K per product
-      const double ldd = double(wv.host_ld[s]);
-      const double t128 = std::ceil(ldd / 128.0);
-      const double tns = std::ceil(ldd / ns_width);
-      const double sym_tiles_ns = ns_width == 256 ? double(sym256_count(int(t128), int(tns))) : t128 * (t128 + 1) / 2;
-      const double tile_ns = 2.0 * 128.0 * ns_width * ldd;
-      const double tile128 = 2.0 * 128.0 * 128.0 * ldd;
-      stats.kernel_exec[KC_TC_NS] += (third ? 3.0 : 2.0) * lp_iters[s] * 3.0 * sym_tiles_ns * tile_ns;
-      const double symt = t128 * (t128 + 1) / 2, fullt = t128 * t128;
-      stats.kernel_exec[KC_TC_REF] += rounds * 3.0 * (2.0 * symt + fullt) * tile128 + cgc[s] * 3.0 * fullt * tile128;
-      if (hp_sliced)
-        stats.kernel_exec[KC_TC_HP] += ((hp_launch_products + hp_pass_full) * fullt + hp_pass_upper * symt) * tile128;
+      // executed MMA work: three MMAs per split product; k_slice_gemm runs whole
+      // 128 x 128 tiles
+      const int ld = wv.host_ld[s];
+      const double full = executed_flops(ld, false), sym = executed_flops(ld, true);
+      stats.kernel_exec[KC_TC_NS] += (third ? 3.0 : 2.0) * lp_iters[s] * 3.0 * sym;
+      stats.kernel_exec[KC_TC_REF] += rounds * 3.0 * (2.0 * sym + full) + cgc[s] * 3.0 * full;
+      if (hp_sliced) {
+        const double t = (ld + 127) / 128, tile = 2.0 * 128.0 * 128.0 * ld;
+        stats.kernel_exec[KC_TC_HP] +=
+            hp_launch_products * full + (hp_pass_full * t * t + hp_pass_upper * t * (t + 1.0) / 2.0) * tile;
+      }
     }
     stats.refine_fallback = fallback_total;
   }
@@ -1878,15 +1875,10 @@ submat_status Plan::backward_wave_tc(size_t wi, const double* K, double mu, cons
       SM_CUDA(cudaStreamSynchronize(st));
       for (double v : part) dn_acc += v;
     }
-    if (timer.on) {  // executed MMA work: three MMAs per split product, tiles x 2 * 128 * 256 * K
-      for (int s = 0; s < wv.count; ++s) {
-        const double ldd = double(wv.host_ld[s]);
-        const int t128 = int(std::ceil(ldd / 128.0)), t256 = int(std::ceil(ldd / 256.0));
-        const double tile = 2.0 * 128.0 * 256.0 * ldd;
-        stats.kernel_exec[KC_TC_ADJ] +=
-            3.0 * tile * (double(sym256_count(t128, t256)) * (steps + updates) + 4.0 * t128 * t256 * steps);
-      }
-    }
+    if (timer.on)  // executed MMA work: three MMAs per split product
+      for (int s = 0; s < wv.count; ++s)
+        stats.kernel_exec[KC_TC_ADJ] += 3.0 * (executed_flops(wv.host_ld[s], true) * (steps + updates) +
+                                               4.0 * executed_flops(wv.host_ld[s], false) * steps);
   }
   int fl = 0;
   SM_TRY(read_flags(st, &fl));
