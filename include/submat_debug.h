@@ -52,8 +52,8 @@ submat_status submat_debug_tc_gemm(int count, int ld, int n, const void* A_hi, c
  *              p < q products carry twice the weight (shift + 1)
  *   per_acc    products per accumulator: 2 (K extents up to 2048) or 1
  *   max_acc    accumulators per launch: 2 (256-wide tiles: paired groups at
- *              most 2^6 apart, combined in 32-bit integers) or 4 (128-wide
- *              tiles: any weights, combined in 64-bit integers)
+ *              most 2^6 apart) or 4 (128-wide tiles: any weights), combined in
+ *              64-bit integers
  *   out        host int32[cap][5] or NULL: one record per slice product,
  *              (launch, accumulator, p, q, shift); the product's weight is
  *              2^shift times 2^(-48) in the int64 sum

@@ -1250,11 +1250,13 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
     // 2^(6 (8 - p - q)) X_p Y_q^T.  sym_pairs (X = Y, symmetric slices): only
     // p <= q, the p < q ones counted twice; the symmetric part of the sum is
     // then the full one.
-    // Products are grouped into exact FP32 accumulators: one level and one
-    // weight each, at most per_acc products.  A launch carries one group, or
-    // two groups whose weights differ by at most 2^6 (two TMEM accumulators,
-    // combined exactly in the epilogue) when their slices fit in <= 6 operand
-    // tiles per stage: fewer launches, so fewer int64 passes.
+    // Where the slices of both fit k_slice_gemm's shared memory (the first round's
+    // do) that is one launch.  Else products are grouped into exact FP32
+    // accumulators: one level and one weight each, at most per_acc products.  A
+    // launch carries up to four groups (two with 256-wide tiles, whose weights
+    // differ by at most 2^6), combined in 64-bit integers in the epilogue, as long
+    // as their slices fit in <= 6 operand tiles per stage: fewer launches, so fewer
+    // int64 passes.
     auto hp_product = [&](const int* xs, int nx, const int* ys, int ny, bool sym_pairs,
                           double* out) -> submat_status {
       if (slice_gemm_fits(nx, ny)) {  // one pass; X X^T from all pairs on its upper tiles
@@ -1299,7 +1301,7 @@ submat_status Plan::sign_mixed(const double* K, double mu, double* D, cudaStream
         p.items = FULL;
         p.nitems = NFULL;
         p.maps = ms->d_maps[wi];
-          p.bn = bn;
+        p.bn = bn;
         p.nbucket = nbk;
         p.nmaps = MS_COUNT * nbk;
         p.na = na; p.nb = nb;

@@ -562,9 +562,9 @@ cudaError_t launch_tc_gemm(const TcGemmParams& p, int grid, cudaStream_t st) {
     return cudaErrorInvalidValue;
   if (p.nacc * bn > p.tmem_cols) return cudaErrorInvalidValue;
   if (p.out_i64) {
-    // full tiles; up to four accumulators of weights 2^i64_shifts[k], combined in 64 bits
-    if (p.sym || p.f16 || p.nacc > 4 || (p.nacc > 2 ? bn != 128 : p.tmem_cols < 2 * p.nacc * bn))
-      return cudaErrorInvalidValue;
+    // full tiles; up to four accumulators of weights 2^i64_shifts[k], combined in 64
+    // bits (double-buffered where TMEM holds two sets, else freed once read)
+    if (p.sym || p.f16 || p.nacc > 4) return cudaErrorInvalidValue;
     for (int k = 0; k < p.nacc; ++k)
       if (p.i64_shifts[k] < 0 || p.i64_shifts[k] > 36) return cudaErrorInvalidValue;
   } else if (p.nacc != 1 || p.tmem_cols < 2 * bn || !(p.out_f32 || p.out_hi)) {
