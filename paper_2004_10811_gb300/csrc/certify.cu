@@ -218,7 +218,9 @@ cudaError_t launch_certify(const WaveDev& w, NsStateDev ns, CertSquare sq, CertL
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // rounding of the computed square, relative to sum_k |X_rk||X_kc|:
-  // FP64 products; FP32 products (ld terms); BF16x3 split products (the
+  // FP64 products (also for residue products, whose operands are rounded to 2^-73 of
+  // at most 2 gx: an entry errs by n^(1/2) 2^-68 gx^2 at most, a row sum by n times
+  // that, less than n 2^-52 gx^2 for n < 2^32); FP32 products (ld terms); BF16x3 split products (the
   // dropped lo*lo term and the pair's own rounding, ~2^-16, FP32 sums of ld
   // terms), doubled for q -> X^2.  FP16x3 split products (mode 3) round to
   // ~2^-21 relative plus 2^-25 absolute per entry (FP16's subnormal step);

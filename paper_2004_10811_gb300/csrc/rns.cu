@@ -989,7 +989,8 @@ cudaError_t launch_rns_rownorm(const WaveDev& w, const double* X, const int* sta
   return cudaGetLastError();
 }
 
-bool rns_route_fits(int max_ld) { return size_t(max_ld) * sizeof(float) <= 200 * 1024; }
+constexpr int ROUTE_SMEM = 200 * 1024;
+bool rns_route_fits(int max_ld) { return size_t(max_ld) * sizeof(float) <= ROUTE_SMEM; }
 
 cudaError_t launch_rns_route(const PatternDev& g, const WaveDev& w, const double* X, int* state, unsigned* least,
                              int* route, int* chains, int nb_max, int max_ld, cudaStream_t st) {
@@ -997,7 +998,8 @@ cudaError_t launch_rns_route(const PatternDev& g, const WaveDev& w, const double
   if (e != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(chains, 0, sizeof(int), st)) != cudaSuccess) return e;
   const int smem = max_ld * int(sizeof(float));
-  if ((e = cudaFuncSetAttribute(k_rns_coupling, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+  if ((e = cudaFuncSetAttribute(k_rns_coupling, cudaFuncAttributeMaxDynamicSharedMemorySize, ROUTE_SMEM)) !=
+      cudaSuccess)
     return e;
   // about eight of the blocks' row sets a CTA
   k_rns_coupling<<<dim3(unsigned(std::max(1, (nb_max + 7) / 8)), unsigned(w.nsub)), 256, size_t(smem), st>>>(
