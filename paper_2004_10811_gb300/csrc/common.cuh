@@ -290,17 +290,6 @@ struct Sum3 {
     two_sum(m, __fadd_rn(e, __fmaf_rn(a, a, -p)), m, e);
     l = __fadd_rn(l, e);
   }
-  __device__ __forceinline__ void add_warp() {  // lane 0 .. 31: the warp's sum
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float xh = __shfl_xor_sync(0xffffffffu, h, o), xm = __shfl_xor_sync(0xffffffffu, m, o);
-      const float xl = __shfl_xor_sync(0xffffffffu, l, o);
-      float e;
-      add(xh);
-      two_sum(m, xm, m, e);
-      l = __fadd_rn(l, __fadd_rn(e, xl));
-    }
-  }
   __device__ __forceinline__ double value() const { return double(h) + (double(m) + double(l)); }
 };
 

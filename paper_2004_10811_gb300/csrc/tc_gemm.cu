@@ -230,6 +230,35 @@ __device__ __forceinline__ void store_mirror(const TcGemmParams& p, int64_t base
   }
 }
 
+// A lane's part of a tile's sum: two to four chunk sums, in a pair (exact for two,
+// else to 2^-48 of the lane's part, less than FP64 loses over the tile).  The warp's
+// sum goes through integers, 25, 23 and 24 bits at a time below the largest part's
+// exponent, by redux instead of FP64 shuffles (a warp's FP64 instruction holds its
+// pipe for 64 clocks).
+struct TileSum {
+  float h = 0.0f, l = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    float e;
+    two_sum(h, x, h, e);
+    l = __fadd_rn(l, e);
+  }
+  __device__ __forceinline__ double warp_sum() const {
+    const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(h) & 0x7F800000u);
+    if (top == 0x7F800000u) return double(__uint_as_float(0x7FC00000u));  // NaN or Inf among them
+    const unsigned e = max(top, 24u << 23);
+    const float up = __uint_as_float((278u << 23) - e), t = h * up, u = l * up;  // |t| < 2^25, |u| <= 3
+    const int a = __float2int_rn(t);
+    const float r = (t - float(a)) * 0x1p23f, s = u * 0x1p23f;
+    const int b0 = __float2int_rn(r), b1 = __float2int_rn(s);
+    const int c = __float2int_rn((r - float(b0)) * 0x1p24f) + __float2int_rn((s - float(b1)) * 0x1p24f);
+    const long long A = __reduce_add_sync(0xffffffffu, a), B = __reduce_add_sync(0xffffffffu, b0 + b1);
+    const long long C = __reduce_add_sync(0xffffffffu, c);
+    // A + B 2^-23 + C 2^-47, at 2^-32, and 2^(e - 151) back
+    const double v = double((A << 32) + (B << 9) + (C >> 15));
+    return v * __longlong_as_double(static_cast<long long>(1023 - 32 - 151 + int(e >> 23)) << 52);
+  }
+};
+
 template <int BN, int MODE, bool F16>
 __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const __grid_constant__ TcGemmParams p) {
   constexpr int TILE_B = BN * BK * 2;  // one BN x 64 BF16 operand tile (B side)
@@ -463,7 +492,7 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const 
         } else {
           const int side = (warp - 2) >> 2;  // chunks side, side + 2, ...
           const bool has_c0 = (p.c0_f32 || p.c0_hi) && p.beta != 0.0f && !p.dot_c0;
-          Sum3 sum;  // the tile's, for res2 or dot_c0
+          TileSum sum;  // for res2 or dot_c0
 #pragma unroll 1
           for (int hc = side; hc < 4 * HALVES; hc += 2) {
             const int h = hc >> 2, c = hc & 3;
@@ -518,14 +547,9 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps(MODE), 1) k_tc_gemm(const 
             if (!p.sym || (diag_sym && c < quarter)) continue;
             store_mirror<F16>(p, base, ld, cg0, item.y * BM + quarter * 32, o, lane, diag_sym && c == quarter);
           }
-          // FP64 instructions hold their pipe for 64 clocks: sums stay in three
-          // FP32 parts up to one conversion per warp
           if (p.res2 || p.dot_c0) {
-            sum.add_warp();
-            if (lane == 0) {
-              const double t = sum.value();
-              if (t != 0.0) atomicAdd(p.res2 ? &p.res2[s] : &p.dot_c0[s], t);
-            }
+            const double t = sum.warp_sum();
+            if (lane == 0 && t != 0.0) atomicAdd(p.res2 ? &p.res2[s] : &p.dot_c0[s], t);
           }
         }
       }
