@@ -277,10 +277,10 @@ struct Sum3 {
   }
   // weight (a + b)^2, weight a power of two and b at most half a unit of a
   __device__ __forceinline__ void add_square(float a, float b, float weight) {
-    const float p = __fmul_rn(a, a);
-    float e = __fmaf_rn(2.0f * a, b, __fmaf_rn(a, a, -p));
-    add(weight * p);
-    two_sum(m, weight * e, m, e);
+    const float p = __fmul_rn(a, a), low = __fmaf_rn(2.0f * a, b, __fmaf_rn(a, a, -p));
+    float e;
+    two_sum(h, weight * p, h, e);
+    two_sum(m, __fmaf_rn(weight, low, e), m, e);
     l = __fadd_rn(l, e);
   }
   __device__ __forceinline__ void add_square(float a) {

@@ -700,16 +700,15 @@ __device__ __forceinline__ void tile_doubles(const Tile& v, int a, int b, int ld
 // 2^23 + a 23-bit piece, as a float, less 2^23: the piece, without a conversion
 __device__ __forceinline__ float piece23(unsigned v) { return __uint_as_float(0x4B000000u | (v & 0x7FFFFFu)) - 8388608.0f; }
 
-// sum += weight n^2, n as an FP32 pair
+// sum += weight n^2, n to 2^-57 as an FP32 pair
 __device__ __forceinline__ void add_square(Sum3& sum, Fix n, float weight) {
   const long long h = n.hi();
-  const float c3 = float(int(h >> 46)) * 0x1p-11f, c2 = piece23(unsigned(h >> 23)) * 0x1p-34f;
-  const float c1 = piece23(unsigned(h)) * 0x1p-57f, c0 = piece23(n.lo()) * 0x1p-73f;
-  float a, e2, e1, e0;
-  two_sum(c3, c2, a, e2);
-  two_sum(a, c1, a, e1);
+  const float c2 = float(int(h >> 46)) * 0x1p-11f, c1 = piece23(unsigned(h >> 23)) * 0x1p-34f;
+  const float c0 = piece23(unsigned(h)) * 0x1p-57f;
+  float a, e1, e0;
+  two_sum(c2, c1, a, e1);
   two_sum(a, c0, a, e0);
-  sum.add_square(a, __fadd_rn(e2, __fadd_rn(e1, e0)), weight);
+  sum.add_square(a, __fadd_rn(e1, e0), weight);
 }
 
 __global__ void __launch_bounds__(256) k_rns_square0(WaveDev w, NsStateDev ns, const unsigned* __restrict__ norm2,
