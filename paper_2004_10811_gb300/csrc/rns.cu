@@ -534,7 +534,9 @@ __device__ __forceinline__ float weight(double x) {
 // Coupling of a submatrix's extracted columns to its rows: the smallest nonzero
 // mean over a block's columns c of (|X| |X|)_rc, over the rows r that the scatter
 // reads, and the smallest nonzero squared norm of a row (a level of its own that the
-// grid would lose); one pass over X for each block column.
+// grid would lose); one pass over X for each block column.  0 where a row's norm is
+// above 2, which the operands' scales do not allow for (values beyond FP32's range,
+// whose bounds saturate, and power estimates far below the spectral radius).
 __global__ void __launch_bounds__(256) k_rns_coupling(PatternDev g, WaveDev w, const double* __restrict__ X,
                                                       const int* __restrict__ state, unsigned* least) {
   extern __shared__ float u[];  // mean of |X_kc| over the block's columns c
@@ -571,6 +573,7 @@ __global__ void __launch_bounds__(256) k_rns_coupling(PatternDev g, WaveDev w, c
         }
         if (a > 0.0f) best = fminf(best, a);
         if (d > 0.0f) best = fminf(best, d);
+        if (d > 4.0f) best = 0.0f;
       }
     }
   }

@@ -79,7 +79,7 @@ cudaError_t launch_rns_rownorm(const WaveDev& w, const double* X, const int* sta
 // (a mean over the block's columns; rows they do not reach at all are exactly zero on
 // either path) goes to the FP64 chains.  An entry's error is about 2^-73 here and
 // 2^-53 of that measure there, so the line is 2^-20 with a margin of four.  Water at
-// a 9 A cutoff lies at 7e-4 and above.
+// a 9 A cutoff lies at 7e-4 and above.  One with a row of norm above 2 goes there too.
 constexpr float RNS_LEAST_COUPLING = 0x1p-18f;
 // the coupling pass holds a row of FP32 in shared memory
 bool rns_route_fits(int max_ld);

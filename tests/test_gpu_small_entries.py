@@ -203,3 +203,20 @@ def test_residual_sums(pkg, beta_mode):
         x = a[np.ix_(idx, idx)] / beta[j]
         want = np.linalg.norm(x @ x - np.eye(len(idx))) / np.sqrt(len(idx))
         assert iters[j] == 1 and abs(resid[j] / want - 1) <= len(idx) ** 0.5 * 2.0 ** -50
+
+
+@pytest.mark.parametrize("beta_mode", [0, 1])
+def test_values_beyond_fp32(pkg, beta_mode):
+    """Entries beyond FP32's range saturate the spectral bound, so the iteration diverges:
+    it says so after one step, and the mu search ends there, instead of running to the
+    step cap on numbers that the grid cannot hold."""
+    import torch
+    m = make_water(20, 4, 4.0, (1, -1.0, -0.3), (3, 0.3, 1.2), seed=2)
+    K = torch.from_numpy(m.vals * 1e100).cuda()
+    with pkg.Plan.from_bsr(m, prec="fp64", beta_mode=beta_mode) as plan:
+        plan.sign(K, 0.0, allow_not_converged=True)
+        s = plan.stats()
+        assert s["not_converged"] == 20 and s["iters_max"] <= 2
+        with pytest.raises(pkg.SubmatError) as e:
+            plan.mu_search(K, 20.0, mu0=0.0, tol=1e-9)
+        assert e.value.name == "NOT_CONVERGED" and "diverged" in str(e.value)
