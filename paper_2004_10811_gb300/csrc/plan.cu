@@ -475,7 +475,7 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
     const size_t ld = size_t(n_max + 63) / 64 * 64;
     const size_t room = std::min(cap, size_t(double(fre) * 0.8));
     for (rns_parts = 1; rns_parts <= (opt.kT > 0.0 ? 1 : 2) && !use_rns; ++rns_parts)
-      use_rns = ld * ld * rns_bytes() <= room && rns_route_fits(int(ld));
+      use_rns = ld * ld * rns_bytes() <= room && rns_route_fits(bs_max);
     --rns_parts;
     if (use_rns) {
       bpe = rns_bytes();
@@ -765,7 +765,7 @@ submat_status Plan::rns_product(size_t wi, int a, int b, RnsSum F, const int* st
 submat_status Plan::rns_route(size_t wi, const double* X, int* state, const int** route, cudaStream_t st) {
   const Wave& wv = waves[wi];
   auto* r = static_cast<RnsState*>(rns);
-  SM_CUDA(launch_rns_route(g, wv.dev, X, state, r->least, r->route, d_active, nb_max, max_ld(wv), st));
+  SM_CUDA(launch_rns_route(g, wv.dev, X, state, r->norm2, r->least, r->route, d_active, bs_max, max_ld(wv), st));
   SM_CUDA(cudaMemcpyAsync(static_cast<int*>(h_pinned) + 1, d_active, sizeof(int), cudaMemcpyDeviceToHost, st));
   if (route) *route = r->route;
   return SUBMAT_OK;
@@ -823,7 +823,6 @@ submat_status Plan::ns_rns(size_t wi, cudaStream_t st) {
   SM_TRY(rns_route(wi, X, ns.state, nullptr, st));
   for (int k = 0; k < opt.max_iter; ++k) {
     if (k == 0) {
-      SM_CUDA(launch_rns_rownorm(wv.dev, X, ns.state, r->norm2, mld, st));
       SM_TRY(product(0, [&](int part) -> submat_status {
         SM_CUDA(launch_rns_convert(wv.dev, X, ns.state, r->norm2, 0, R[0], RnsFix{}, mld, st, rns_parts, part));
         return SUBMAT_OK;

@@ -503,81 +503,96 @@ __device__ __forceinline__ int norm_shift(unsigned bits) {
   return e >= 0 ? (e + 1) / 2 : -(-e / 2);
 }
 
-__global__ void __launch_bounds__(256) k_rns_rownorm(WaveDev w, const double* __restrict__ X,
-                                                     const int* __restrict__ state, unsigned* norm2) {
-  const int s = blockIdx.y;
-  if (state && state[s] == ST_DONE) return;
-  const int ld = w.ld[s], n = w.n[s];
-  const double* Xs = X + w.off[s];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float best = 0.0f;
-  for (int r = blockIdx.x * 8 + warp; r < n; r += gridDim.x * 8) {
-    float acc = 0.0f;
-    for (int c = 2 * lane; c < ld; c += 64) {
-      const double2 v = *reinterpret_cast<const double2*>(Xs + int64_t(r) * ld + c);
-      const float a = d2f_trunc(v.x), b = d2f_trunc(v.y);
-      acc = fmaf(a, a, acc);
-      acc = fmaf(b, b, acc);
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    best = fmaxf(best, acc);
-  }
-  // sums of truncated squares: the margin covers truncation and rounding (ld <= 32768)
-  if (lane == 0 && best > 0.0f) atomicMax(&norm2[s], __float_as_uint(best * 1.01f));
-}
-
 // |x| as FP32, nonzero where x is (a floor that keeps products of two in range)
 __device__ __forceinline__ float weight(double x) {
   return x == 0.0 ? 0.0f : fmaxf(fabsf(d2f_trunc(x)), 0x1p-60f);
 }
 
-// Coupling of a submatrix's extracted columns to its rows: the smallest nonzero
-// mean over a block's columns c of (|X| |X|)_rc, over the rows r that the scatter
-// reads, and the smallest nonzero squared norm of a row (a level of its own that the
-// grid would lose); one pass over X for each block column.  0 where a row's norm is
-// above 2, which the operands' scales do not allow for (values beyond FP32's range,
-// whose bounds saturate, and power estimates far below the spectral radius).
+__device__ __forceinline__ float warp_sum(float a) {
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
+// Squared row norms: the largest into norm2, the smallest nonzero one into least (a
+// level of its own that the grid would lose).  least becomes 0 where a norm is above
+// 2, which the operands' scales do not allow for (values beyond FP32's range, whose
+// bounds saturate, and power estimates far below the spectral radius).
+__global__ void __launch_bounds__(256) k_rns_rownorm(WaveDev w, const double* __restrict__ X,
+                                                     const int* __restrict__ state, unsigned* norm2, unsigned* least) {
+  const int s = blockIdx.y;
+  if (state && state[s] == ST_DONE) return;
+  const int ld = w.ld[s], n = w.n[s];
+  const double* Xs = X + w.off[s];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float most = 0.0f, few = __uint_as_float(0x7F7FFFFFu);
+  for (int r = blockIdx.x * 8 + warp; r < n; r += gridDim.x * 8) {
+    float acc = 0.0f;
+    for (int c = 2 * lane; c < ld; c += 64) {
+      const double2 v = *reinterpret_cast<const double2*>(Xs + int64_t(r) * ld + c);
+      const float a = weight(v.x), b = weight(v.y);
+      acc = fmaf(a, a, acc);
+      acc = fmaf(b, b, acc);
+    }
+    acc = warp_sum(acc);
+    most = fmaxf(most, acc);
+    if (acc > 0.0f) few = fminf(few, acc);
+  }
+  if (most > 4.0f) few = 0.0f;
+  // sums of truncated squares: the margin covers truncation and rounding (ld <= 32768)
+  if (lane == 0 && most > 0.0f) {
+    atomicMax(&norm2[s], __float_as_uint(most * 1.01f));
+    atomicMin(&least[s], __float_as_uint(few));
+  }
+}
+
+// Coupling of a submatrix's extracted columns to its rows: the smallest nonzero mean
+// over a block's columns c of (|X| |X|)_rc, over the rows r that the scatter reads.
+// The term |X_rc| |X_cc| alone, a lower bound, decides nearly all of them with one
+// read of the extracted columns; where it does not, the whole sum is formed.
 __global__ void __launch_bounds__(256) k_rns_coupling(PatternDev g, WaveDev w, const double* __restrict__ X,
                                                       const int* __restrict__ state, unsigned* least) {
-  extern __shared__ float u[];  // mean of |X_kc| over the block's columns c
+  extern __shared__ float diag[];  // |X_cc| of the block's columns
   const int s = blockIdx.y;
   if (state && state[s] == ST_DONE) return;
   const int ld = w.ld[s], n = w.n[s], q = w.sub[s];
   const double* Xs = X + w.off[s];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = g.mp ? g.mp[q] : 0, m1 = g.mp ? g.mp[q + 1] : 1;
-  float best = __uint_as_float(0x7F7FFFFFu);
-  for (int mi = m0; mi < m1; ++mi) {
-    const int j = g.mp ? g.mcol[mi] : q;
-    const int64_t k0 = g.mp ? g.mkoff[mi] : g.koff[j];
-    const int b = g.bs[j];
+  const volatile unsigned* known = least;
+  int64_t k0 = 0;
+  int b = 0;
+  auto row = [&](int r) {
+    if (__uint_as_float(__shfl_sync(0xffffffffu, known[s], 0)) < RNS_LEAST_COUPLING) return;  // decided
+    const double* xr = Xs + int64_t(r) * ld;
+    float a = 0.0f;
+    for (int c = lane; c < b; c += 32) a = fmaf(weight(xr[k0 + c]), diag[c], a);
+    a = warp_sum(a) / float(b);
+    if (a >= RNS_LEAST_COUPLING) return;
+    a = 0.0f;
+    for (int c = 0; c < b; ++c)
+      for (int k = lane; k < n; k += 32) a = fmaf(weight(xr[k]), weight(Xs[(k0 + c) * ld + k]), a);
+    a = warp_sum(a) / float(b);
+    if (lane == 0 && a > 0.0f) atomicMin(&least[s], __float_as_uint(a));
+  };
+  auto columns = [&](int j, int64_t at) {
+    k0 = at;
+    b = g.bs[j];
     __syncthreads();
-    for (int c = threadIdx.x; c < n; c += 256) {
-      float a = 0.0f;
-      for (int t = 0; t < b; ++t) a += weight(Xs[(k0 + t) * ld + c]);
-      u[c] = a / float(b);
-    }
+    for (int c = threadIdx.x; c < b; c += 256) diag[c] = weight(Xs[(k0 + c) * ld + k0 + c]);
     __syncthreads();
+  };
+  if (!g.mp) {  // one block column: every row
+    columns(q, g.koff[q]);
+    for (int r = blockIdx.x * 8 + warp; r < n; r += gridDim.x * 8) row(r);
+    return;
+  }
+  for (int mi = g.mp[q]; mi < g.mp[q + 1]; ++mi) {
+    const int j = g.mcol[mi];
+    columns(j, g.mkoff[mi]);
     for (int64_t p = g.row_ptr[j] + blockIdx.x; p < g.row_ptr[j + 1]; p += gridDim.x) {
-      const int r0 = g.mp ? g.dloc[g.tpos[p]] : g.locoff[p], nr = g.bs[g.col[p]];
-      for (int t = warp; t < nr; t += 8) {
-        float a = 0.0f, d = 0.0f;
-        for (int c = lane; c < n; c += 32) {
-          const float x = weight(Xs[int64_t(r0 + t) * ld + c]);
-          a = fmaf(x, u[c], a);
-          d = fmaf(x, x, d);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          a += __shfl_xor_sync(0xffffffffu, a, o);
-          d += __shfl_xor_sync(0xffffffffu, d, o);
-        }
-        if (a > 0.0f) best = fminf(best, a);
-        if (d > 0.0f) best = fminf(best, d);
-        if (d > 4.0f) best = 0.0f;
-      }
+      const int r0 = g.dloc[g.tpos[p]], nr = g.bs[g.col[p]];
+      for (int t = warp; t < nr; t += 8) row(r0 + t);
     }
   }
-  if (lane == 0) atomicMin(&least[s], __float_as_uint(best));
 }
 
 // route[s]: ST_DONE for the chains, ST_ACTIVE for the residues.  With state, an
@@ -982,30 +997,23 @@ cudaError_t launch_rns_gemm(RnsGemmParams p, int nsm, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_rns_rownorm(const WaveDev& w, const double* X, const int* state, unsigned* norm2, int max_ld,
-                               cudaStream_t st) {
+constexpr int ROUTE_SMEM = 200 * 1024;
+bool rns_route_fits(int bs_max) { return size_t(bs_max) * sizeof(float) <= ROUTE_SMEM; }
+
+cudaError_t launch_rns_route(const PatternDev& g, const WaveDev& w, const double* X, int* state, unsigned* norm2,
+                             unsigned* least, int* route, int* chains, int bs_max, int max_ld, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(norm2, 0, sizeof(unsigned) * size_t(w.nsub), st);
   if (e != cudaSuccess) return e;
-  k_rns_rownorm<<<dim3(unsigned(std::min((max_ld + 31) / 32, 64)), unsigned(w.nsub)), 256, 0, st>>>(w, X, state, norm2);
-  count_launch();
-  return cudaGetLastError();
-}
-
-constexpr int ROUTE_SMEM = 200 * 1024;
-bool rns_route_fits(int max_ld) { return size_t(max_ld) * sizeof(float) <= ROUTE_SMEM; }
-
-cudaError_t launch_rns_route(const PatternDev& g, const WaveDev& w, const double* X, int* state, unsigned* least,
-                             int* route, int* chains, int nb_max, int max_ld, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(least, 0x7F, sizeof(unsigned) * size_t(w.nsub), st);
-  if (e != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(least, 0x7F, sizeof(unsigned) * size_t(w.nsub), st)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(chains, 0, sizeof(int), st)) != cudaSuccess) return e;
-  const int smem = max_ld * int(sizeof(float));
+  const dim3 grid(unsigned(std::min((max_ld + 31) / 32, 64)), unsigned(w.nsub));
+  k_rns_rownorm<<<grid, 256, 0, st>>>(w, X, state, norm2, least);
+  count_launch();
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_rns_coupling, cudaFuncAttributeMaxDynamicSharedMemorySize, ROUTE_SMEM)) !=
       cudaSuccess)
     return e;
-  // about eight of the blocks' row sets a CTA
-  k_rns_coupling<<<dim3(unsigned(std::max(1, (nb_max + 7) / 8)), unsigned(w.nsub)), 256, size_t(smem), st>>>(
-      g, w, X, state, least);
+  k_rns_coupling<<<grid, 256, size_t(bs_max) * sizeof(float), st>>>(g, w, X, state, least);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_rns_route<<<(w.nsub + 255) / 256, 256, 0, st>>>(w.nsub, least, route, state, chains);

@@ -72,22 +72,20 @@ struct RnsGemmParams {
 int rns_split(int ntiles, int nmod, int nsm);
 cudaError_t launch_rns_gemm(RnsGemmParams p, int nsm, cudaStream_t st);
 
-// Largest row 2-norm squared of X per submatrix (bits of a float) into norm2.
-cudaError_t launch_rns_rownorm(const WaveDev& w, const double* X, const int* state, unsigned* norm2, int max_ld,
-                               cudaStream_t st);
 // A submatrix whose extracted columns reach a row with less than this in (|X| |X|)
 // (a mean over the block's columns; rows they do not reach at all are exactly zero on
 // either path) goes to the FP64 chains.  An entry's error is about 2^-73 here and
 // 2^-53 of that measure there, so the line is 2^-20 with a margin of four.  Water at
 // a 9 A cutoff lies at 7e-4 and above.  One with a row of norm above 2 goes there too.
 constexpr float RNS_LEAST_COUPLING = 0x1p-18f;
-// the coupling pass holds a row of FP32 in shared memory
-bool rns_route_fits(int max_ld);
+// the coupling pass holds a block's diagonal in FP32 in shared memory
+bool rns_route_fits(int bs_max);
 // route[s] = ST_DONE for submatrices of the chains, else ST_ACTIVE, and their number
 // into chains.  With state, submatrices not active are left out and those of the
-// chains are held (ST_DONE) until launch_rns_resume.
-cudaError_t launch_rns_route(const PatternDev& g, const WaveDev& w, const double* X, int* state, unsigned* least,
-                             int* route, int* chains, int nb_max, int max_ld, cudaStream_t st);
+// chains are held (ST_DONE) until launch_rns_resume.  norm2: the largest row 2-norm
+// squared of X per submatrix (bits of a float).
+cudaError_t launch_rns_route(const PatternDev& g, const WaveDev& w, const double* X, int* state, unsigned* norm2,
+                             unsigned* least, int* route, int* chains, int bs_max, int max_ld, cudaStream_t st);
 cudaError_t launch_rns_resume(const WaveDev& w, const int* route, int* state, cudaStream_t st);
 
 // Residues of X 2^-sh for a complete FP64 matrix; sh from norm2 (the smallest
