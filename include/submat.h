@@ -97,7 +97,7 @@ typedef struct {
                                   for FP64 plans, or what the largest submatrix needs).  Bytes
                                   per entry of a wave's padded submatrices: FP64 98 (72 where
                                   that is all that fits one submatrix; 24 below that), with
-                                  kT > 0 198 (96 below that); submat_sign_backward has its own
+                                  kT > 0 198 (162, 96 below that); submat_sign_backward has its own
                                   workspace under the same cap */
   int refine_rounds;           /* mixed path: correction rounds; 0 selects 1.  With one
                                   round a submatrix is accepted when its Lyapunov solve

@@ -384,9 +384,11 @@ submat_status Plan::fermi_wave(Wave& wv, int wi, const double* K, double mu, dou
   const bool residues = wi >= 0;  // FP64 forward only
   if (residues) {
     const RnsSum F = fermi_rns_sum();  // in A's memory, which has served its purpose
-    SM_CUDA(launch_rns_convert(wv.dev, reinterpret_cast<double*>(odd), nullptr, nullptr, 0, rns_residues(1), RnsFix{},
-                               max_ld(wv), st));
-    SM_TRY(rns_product(size_t(wi), 1, 1, F, nullptr, st));
+    for (int part = 0; part < rns_parts; ++part) {
+      SM_CUDA(launch_rns_convert(wv.dev, reinterpret_cast<double*>(odd), nullptr, nullptr, 0, rns_residues(1),
+                                 RnsFix{}, max_ld(wv), st, rns_parts, part));
+      SM_TRY(rns_product(size_t(wi), 1, 1, F, nullptr, st, part));
+    }
     SM_CUDA(launch_rns_cheb2(wv.dev, F, reinterpret_cast<double*>(T2), max_ld(wv), st));
     ++products;
   } else {
@@ -501,7 +503,8 @@ RnsSum Plan::fermi_rns_sum() const {
 // and T_2 in FP64, to p(X) in FP64 in the first Clenshaw buffer; submatrices of the
 // chains are left as they are.  Every T_k has norm 1 or less; the Clenshaw terms
 // move as b_j 2^-e (fermi_clenshaw_exponent).  Residue set 0 holds the factor that
-// stays (T_2, then Y), set 1 the one that each pass renews.
+// stays (T_2, then Y), set 1 the one that each pass renews; with the moduli in two
+// parts, each product takes both from the fixed-point matrices instead.
 // 240 submatrices of 219-384 dims (blocks of 13, 5 and 5 functions, kT 0.05): a
 // build takes 33.6 ms, 15.4 of them in the products, against 574 ms with the FP64
 // SIMT GEMM.
@@ -517,49 +520,58 @@ submat_status Plan::fermi_rns(int wi, const FermiPoly& P, const int* route, int*
   };
   auto odd = [&](int q) { return fix(q); };
   const RnsFix T2 = fix(H);
+  const bool whole = rns_parts == 1;
   __nv_bfloat16* R[2] = {rns_residues(0), rns_residues(1)};
-  auto product = [&]() -> submat_status {  // F = (set 0) (set 1)
+  __nv_bfloat16* made[2] = {whole ? R[0] : nullptr, whole ? R[1] : nullptr};  // written by the passes
+  auto product = [&](const RnsFix& a, const RnsFix& b) -> submat_status {  // F = (set 0) (set 1) = a b
     ++*products;
-    return rns_product(size_t(wi), 0, 1, F, route, st);
+    for (int part = 0; part < rns_parts; ++part) {
+      if (!whole) {
+        SM_CUDA(launch_rns_spread(wv.dev, route, a, R[0], mld, st, part));
+        SM_CUDA(launch_rns_spread(wv.dev, route, b, R[1], mld, st, part));
+      }
+      SM_TRY(rns_product(size_t(wi), 0, 1, F, route, st, part));
+    }
+    return SUBMAT_OK;
   };
   auto dbl = [](const RnsFix& x) { return reinterpret_cast<double*>(x.hi); };
-  SM_CUDA(launch_rns_convert(wv.dev, dbl(odd(0)), route, nullptr, 0, R[1], odd(0), mld, st));
-  SM_CUDA(launch_rns_convert(wv.dev, dbl(T2), route, nullptr, 0, R[0], T2, mld, st));
+  SM_CUDA(launch_rns_convert(wv.dev, dbl(odd(0)), route, nullptr, 0, made[1], odd(0), mld, st));
+  SM_CUDA(launch_rns_convert(wv.dev, dbl(T2), route, nullptr, 0, made[0], T2, mld, st));
   RnsCheb c{};
   c.state = route;
   c.F = F;
   c.twice = 1;
-  c.R = R[1];
+  c.R = made[1];
   for (int q = 1; q < H; ++q) {  // T_{2q+1} = 2 T_2 T_{2q-1} - T_{2q-3}, T_{-1} = T_1
-    SM_TRY(product());
+    SM_TRY(product(T2, odd(q - 1)));
     c.sub = odd(std::max(0, q - 2));
     c.C = odd(q);
     if (q == H - 1) c.R = nullptr;
     SM_CUDA(launch_rns_cheb(wv.dev, c, mld, st));
   }
-  for (int i = 0; i < 2; ++i) {  // residues of -T_9 and -T_7
+  for (int i = 0; whole && i < 2; ++i) {  // residues of -T_9 and -T_7
     RnsCheb t{};
     t.state = route;
     t.sub = odd(H / 2 - i);
     t.R = R[i];
     SM_CUDA(launch_rns_cheb(wv.dev, t, mld, st));
   }
-  SM_TRY(product());  // Y = T_16 = 2 T_9 T_7 - T_2
+  SM_TRY(product(odd(H / 2), odd(H / 2 - 1)));  // Y = T_16 = 2 T_9 T_7 - T_2
   c.sub = T2;
   c.C = T2;
-  c.R = R[0];
+  c.R = made[0];
   SM_CUDA(launch_rns_cheb(wv.dev, c, mld, st));
   // giant steps: b_j = R_j + 2 Y b_{j+1} - b_{j+2}, p = R_0 + Y b_1 - b_2
   c = RnsCheb{};
   c.state = route;
   c.odd = odd(0);
   c.stride = E;
-  c.R = R[1];
+  c.R = made[1];
   for (int j = P.blocks - 1; j >= 0; --j) {
     const RnsFix W = fix(H + 1 + (j & 1));  // b_{j+2}'s place
     for (int q = 0; q < H; ++q) c.coef[q] = std::llrint(std::ldexp(P.r[size_t(j) * H + q], RNS_COEF - e));
     if (j < P.blocks - 1) {
-      SM_TRY(product());
+      SM_TRY(product(T2, fix(H + 1 + ((j + 1) & 1))));
       c.F = F;
     }
     c.twice = j > 0;

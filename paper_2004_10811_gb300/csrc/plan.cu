@@ -463,8 +463,8 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
   SM_CUDA(cudaMemGetInfo(&fre, &tot));
   if (cap == 0) cap = size_t(double(fre) * 0.8);
   if (opt.prec == SUBMAT_FP64) {
-    // Residue products (98 B per element, 198 B at finite temperature; 72 B with
-    // the moduli in two parts) wherever the largest submatrix fits the workspace
+    // Residue products (98 B per element, 198 B at finite temperature; 72 and 162 B
+    // with the moduli in two parts) wherever the largest submatrix fits the workspace
     // that way; the SIMT GEMM (24 B and 96 B) below that.  They are 15x faster
     // where the waves fill the chip (216 submatrices of 420-480 dims in one wave:
     // 28.8 against 425.8 ms).  A cap of a few submatrices holds four times as many
@@ -474,7 +474,7 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
     // plan's cap does not change its arithmetic.
     const size_t ld = size_t(n_max + 63) / 64 * 64;
     const size_t room = std::min(cap, size_t(double(fre) * 0.8));
-    for (rns_parts = 1; rns_parts <= (opt.kT > 0.0 ? 1 : 2) && !use_rns; ++rns_parts)
+    for (rns_parts = 1; rns_parts <= 2 && !use_rns; ++rns_parts)
       use_rns = ld * ld * rns_bytes() <= room && rns_route_fits(bs_max);
     --rns_parts;
     if (use_rns) {

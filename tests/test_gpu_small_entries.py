@@ -220,3 +220,25 @@ def test_values_beyond_fp32(pkg, beta_mode):
         with pytest.raises(pkg.SubmatError) as e:
             plan.mu_search(K, 20.0, mu0=0.0, tol=1e-9)
         assert e.value.name == "NOT_CONVERGED" and "diverged" in str(e.value)
+
+
+@pytest.mark.parametrize("kT", [0.05, 0.3])
+def test_fermi_moduli_in_two_parts(pkg, kT):
+    """A workspace that holds 162 to 198 bytes for each entry of the largest submatrix:
+    the residue sets hold half of the moduli at a time, with the same bits as a result
+    (one block column a plan, so that the scale is the submatrix's own)."""
+    import torch
+    m = make_water(40, 6, 5.0, (2, -1.0, -0.3), (4, 0.3, 1.0), seed=21)
+    K = torch.from_numpy(m.vals).cuda()
+    ld = (6 * int(np.diff(m.row_ptr).max()) + 63) // 64 * 64
+    for j in (3, 30):
+        kw = dict(prec="fp64", kT=kT, columns=(j, j + 1), timing=True)
+        got = []
+        for cap in (0, 163 * ld * ld):
+            with pkg.Plan.from_bsr(m, workspace_cap_bytes=cap, **kw) as plan:
+                got.append(plan.sign(K, 0.0, out=torch.zeros_like(K)))
+                s = plan.stats()
+            assert s["kernel_launches"][RESIDUES] > 0 == s["kernel_launches"][SIMT]
+        # 9 baby products and the giant steps, each in two launches
+        assert s["kernel_launches"][RESIDUES] == 2 * s["iters_max"]
+        assert torch.equal(got[0], got[1]) and float(got[0].abs().max()) > 0.1
