@@ -506,7 +506,7 @@ RnsSum Plan::fermi_rns_sum() const {
 // stays (T_2, then Y), set 1 the one that each pass renews; with the moduli in two
 // parts, each product takes both from the fixed-point matrices instead.
 // 240 submatrices of 219-384 dims (blocks of 13, 5 and 5 functions, kT 0.05): a
-// build takes 33.6 ms, 15.4 of them in the products, against 574 ms with the FP64
+// build takes 33.4 ms, 15.4 of them in the products, against 574 ms with the FP64
 // SIMT GEMM.
 submat_status Plan::fermi_rns(int wi, const FermiPoly& P, const int* route, int* products, cudaStream_t st) {
   constexpr int H = kFermiBaby / 2;

@@ -467,7 +467,7 @@ submat_status Plan::build(int nblk_, const int32_t* bs_, const int64_t* rp_, con
     // with the moduli in two parts) wherever the largest submatrix fits the workspace
     // that way; the SIMT GEMM (24 B and 96 B) below that.  They are 15x faster
     // where the waves fill the chip (216 submatrices of 420-480 dims in one wave:
-    // 28.8 against 425.8 ms).  A cap of a few submatrices holds four times as many
+    // 28.6 against 425.8 ms).  A cap of a few submatrices holds four times as many
     // of the SIMT GEMM's, and each wave costs its launches: one residue wave per
     // submatrix takes 548 ms there (54 SIMT waves: ~560) and for 125 of 64 dims 109
     // (32 SIMT waves: ~52).  The line stays at what fits all the same, so that a

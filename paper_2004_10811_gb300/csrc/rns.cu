@@ -136,7 +136,7 @@ __device__ __forceinline__ void fold_guard(unsigned long long& f, uint32_t& g, u
 // clock, and by a tenth by the guard sums' way through TMEM (16.4 against 14.9 ms
 // for 18 products without it; loading a chunk ahead of the one in work: 16.1).
 // Measured on 216 submatrices of 420-480 dims: 0.89 ms a product, against
-// 23.5 ms for the FP64 SIMT GEMM; a whole build 28.8 against 425.9 ms.
+// 23.5 ms for the FP64 SIMT GEMM; a whole build 28.6 against 425.9 ms.
 __global__ void __launch_bounds__(THREADS, 1) k_rns_gemm(const __grid_constant__ RnsGemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
