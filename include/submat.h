@@ -63,10 +63,9 @@ typedef enum {
                                     fixed-point products on a 2^-73 grid (the iterates have norm
                                     1), exact in residue arithmetic on the tensor cores.  FP64
                                     multiply-add chains on the SIMT GEMM, about 15x slower,
-                                    evaluate the submatrices whose extracted columns couple to
-                                    some row by less than 2^-18 but not 0 (at kT > 0: their
-                                    shares of a wave), where the grid is coarser than FP64, and
-                                    plans whose workspace is too small for the residues */
+                                    evaluate the submatrices with less than 2^-18, but not 0, in
+                                    an extracted entry of |X_0|^2, where the grid is coarser than
+                                    FP64, and plans whose workspace is too small for the residues */
   SUBMAT_FP32 = 1,               /* Newton-Schulz in FP32 (no refinement) */
   SUBMAT_MIXED_BF16_REFINE = 2   /* tensor-core Newton-Schulz on FP16 (hi, lo) pairs, then an
                                     FP64-anchored correction from BF16 and exact sliced

@@ -545,10 +545,11 @@ __global__ void __launch_bounds__(256) k_rns_rownorm(WaveDev w, const double* __
   }
 }
 
-// Coupling of a submatrix's extracted columns to its rows: the smallest nonzero mean
-// over a block's columns c of (|X| |X|)_rc, over the rows r that the scatter reads.
-// The term |X_rc| |X_cc| alone, a lower bound, decides nearly all of them with one
-// read of the extracted columns; where it does not, the whole sum is formed.
+// Coupling of a submatrix's extracted columns to its rows: whether some entry that
+// the scatter reads has 0 < (|X| |X|)_rc < RNS_LEAST_COUPLING (into least).  A warp
+// takes 32 entries of a row: the term |X_rc| |X_cc| alone, a lower bound, decides
+// nearly all of them with one read of the extracted columns; where it does not, the
+// sum is formed, from the columns' own rows on and only until it is large enough.
 __global__ void __launch_bounds__(256) k_rns_coupling(PatternDev g, WaveDev w, const double* __restrict__ X,
                                                       const int* __restrict__ state, unsigned* least) {
   extern __shared__ float diag[];  // |X_cc| of the block's columns
@@ -561,17 +562,28 @@ __global__ void __launch_bounds__(256) k_rns_coupling(PatternDev g, WaveDev w, c
   int64_t k0 = 0;
   int b = 0;
   auto row = [&](int r) {
-    if (__uint_as_float(__shfl_sync(0xffffffffu, known[s], 0)) < RNS_LEAST_COUPLING) return;  // decided
     const double* xr = Xs + int64_t(r) * ld;
-    float a = 0.0f;
-    for (int c = lane; c < b; c += 32) a = fmaf(weight(xr[k0 + c]), diag[c], a);
-    a = warp_sum(a) / float(b);
-    if (a >= RNS_LEAST_COUPLING) return;
-    a = 0.0f;
-    for (int c = 0; c < b; ++c)
-      for (int k = lane; k < n; k += 32) a = fmaf(weight(xr[k]), weight(Xs[(k0 + c) * ld + k]), a);
-    a = warp_sum(a) / float(b);
-    if (lane == 0 && a > 0.0f) atomicMin(&least[s], __float_as_uint(a));
+    for (int c0 = 0; c0 < b; c0 += 32) {
+      if (__uint_as_float(__shfl_sync(0xffffffffu, known[s], 0)) < RNS_LEAST_COUPLING) return;  // decided
+      const int c = c0 + lane;
+      const bool mine = c < b;
+      if (__all_sync(0xffffffffu, !mine || weight(xr[k0 + c]) * diag[c] >= RNS_LEAST_COUPLING)) continue;
+      const int chunks = (n + 31) / 32, first = int(k0 + c0) / 32;
+      float a = 0.0f;
+      for (int t = 0; t < chunks; ++t) {
+        const int k1 = (first + t) % chunks * 32;
+        const float x = k1 + lane < n ? weight(xr[k1 + lane]) : 0.0f;
+        unsigned some = __ballot_sync(0xffffffffu, x != 0.0f);
+        if (some == 0) continue;
+        for (; some; some &= some - 1) {
+          const int k = __ffs(int(some)) - 1;
+          const float xk = __shfl_sync(0xffffffffu, x, k);
+          if (mine) a = fmaf(xk, weight(Xs[int64_t(k1 + k) * ld + k0 + c]), a);
+        }
+        if (__all_sync(0xffffffffu, !mine || a >= RNS_LEAST_COUPLING)) break;
+      }
+      if (mine && a > 0.0f && a < RNS_LEAST_COUPLING) atomicMin(&least[s], __float_as_uint(a));
+    }
   };
   auto columns = [&](int j, int64_t at) {
     k0 = at;

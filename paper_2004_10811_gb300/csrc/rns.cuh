@@ -72,11 +72,11 @@ struct RnsGemmParams {
 int rns_split(int ntiles, int nmod, int nsm);
 cudaError_t launch_rns_gemm(RnsGemmParams p, int nsm, cudaStream_t st);
 
-// A submatrix whose extracted columns reach a row with less than this in (|X| |X|)
-// (a mean over the block's columns; rows they do not reach at all are exactly zero on
-// either path) goes to the FP64 chains.  An entry's error is about 2^-73 here and
-// 2^-53 of that measure there, so the line is 2^-20 with a margin of four.  Water at
-// a 9 A cutoff lies at 7e-4 and above.  One with a row of norm above 2 goes there too.
+// A submatrix with less than this, but not 0, in (|X| |X|)_rc of an extracted entry, or
+// in a row's squared norm, goes to the FP64 chains (an entry that is 0 there is exactly
+// zero on either path).  An entry's error is about 2^-73 here and 2^-53 of that measure
+// there, so the line is 2^-20 with a margin of four.  Water at a 9 A cutoff lies at
+// 6e-4 and above.  One with a row of norm above 2 goes there too.
 constexpr float RNS_LEAST_COUPLING = 0x1p-18f;
 // the coupling pass holds a block's diagonal in FP32 in shared memory
 bool rns_route_fits(int bs_max);

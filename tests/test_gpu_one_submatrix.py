@@ -97,3 +97,27 @@ def test_fermi_levels(pkg, kT):
         N *= 2
     want = 1.0 / (1.0 + np.exp(x / kT))
     assert np.max(np.abs(D - want)) <= 2e-13 + 2 * N ** 0.5 * 2.0 ** -53 * N / 4
+
+
+@pytest.mark.parametrize("kT", [0.0, 0.5])
+def test_fp64_many_chunks(pkg, kT):
+    """3300 dims: four exact chunks of each of 19 moduli, more phases (76) than the guard
+    sums of k_rns_gemm take without being folded.  A = Q w Q^T with Q known to n 2^-53;
+    bounds as above."""
+    import torch
+    n = 3300
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, _ = torch.linalg.qr(torch.randn(n, n, generator=g, device="cuda", dtype=torch.float64))
+    w = 0.2 + 0.8 * torch.rand(n, generator=g, device="cuda", dtype=torch.float64)
+    w[: n // 2] *= -1.0
+    a = (q * w) @ q.T
+    a = 0.5 * (a + a.T)
+    want = (q * (torch.sigmoid(-w / kT) if kT else (w < 0).double())) @ q.T
+    with pkg.Plan(np.array([n], np.int32), np.array([0, 1], np.int64), np.array([0], np.int32), prec="fp64", kT=kT,
+                  timing=True) as plan:
+        D = plan.sign(a.flatten().contiguous(), 0.0).reshape(n, n)
+        s = plan.stats()
+    assert s["kernel_launches"][7] > 0 == s["kernel_launches"][2]
+    err = float((D - want).abs().max())
+    assert err <= n * 25 * 3e-16 / 0.2 if not kT else 2e-13 + n * 3e-16 * (256 / (4 * kT) + 16)
+    assert err <= 1e-12

@@ -95,6 +95,18 @@ def test_weak_coupling(pkg, eps):
         assert not chains or eps < 1e-3
 
 
+@pytest.mark.parametrize("eps", [1e-2, 1e-4, 1e-8, 1e-12, 1e-25])
+def test_weak_coupling_inside_a_block(pkg, eps):
+    """The same pair of clusters as one block of 24 functions."""
+    m = pairs([eps])
+    a = dense(m, 0)
+    one = BSRMatrix(np.array([2 * M], np.int32), np.array([0, 1]), np.array([0], np.int32), a.ravel().copy())
+    D, s = run(pkg, one)
+    want = -0.5 * sign_long(a)[:M, M:]
+    e = np.linalg.norm((D.reshape(2 * M, 2 * M)[:M, M:] - want).astype(float)) / np.linalg.norm(want.astype(float))
+    assert e <= BOUND and (s["kernel_launches"][SIMT] > 0) == (eps < 1e-5)
+
+
 @pytest.mark.parametrize("eps", [1e-2, 1e-4, 1e-6, 1e-10, 1e-16])
 @pytest.mark.parametrize("kT", [0.05, 0.3])
 def test_weak_coupling_fermi(pkg, eps, kT):
