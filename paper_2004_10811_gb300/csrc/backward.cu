@@ -154,7 +154,7 @@ template <typename T>
 cudaError_t launch_bwd_scatter_add(const PatternDev& g, const Wave& wv, int nb_max, const T* E, double* Kbar,
                                    cudaStream_t st) {
   const size_t smem = size_t(3 * nb_max + 1) * sizeof(int);
-  if (smem > 48 * 1024) {
+  if (smem > kSmemByDefault) {
     const cudaError_t e = cudaFuncSetAttribute(k_bwd_scatter_add<T>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
@@ -275,7 +275,7 @@ submat_status Plan::backward_wave(Wave& wv, const double* K, double mu, const do
     }
     if (pass == 0) {
       const size_t smem = size_t(3 * nb_max + 1) * sizeof(int);
-      if (smem > 48 * 1024)
+      if (smem > kSmemByDefault)
         SM_CUDA(cudaFuncSetAttribute(k_bwd_scatter_add<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
       k_bwd_scatter_add<T><<<wv.n_gather, 256, smem, st>>>(
           g, wv.dev, wv.gather_items, Ed[cur], Kbar);

@@ -42,6 +42,10 @@ long long launch_count();
     if (s_ != SUBMAT_OK) return s_;              \
   } while (0)
 
+// Dynamic shared memory up to this needs no attribute: 48 KB less room for a kernel's
+// own static arrays, which count towards the same default limit.
+constexpr size_t kSmemByDefault = 40 * 1024;
+
 // Device status word bits (plan->d_flags[0]).
 enum : int { FLAG_NONFINITE = 1, FLAG_TIMEOUT = 2, FLAG_DIVERGED = 4, FLAG_BOUNDS = 8 };
 

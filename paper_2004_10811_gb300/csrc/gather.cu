@@ -301,7 +301,7 @@ cudaError_t launch_scatter_members(const PatternDev& g, const WaveDev& w, NsStat
                                    double* sqpart) {
   if (w.nsub <= 0) return cudaSuccess;
   const size_t smem = size_t(3 * nbj_max + 1) * sizeof(int);
-  if (smem > 48 * 1024) {
+  if (smem > kSmemByDefault) {
     const cudaError_t e = cudaFuncSetAttribute(k_scatter_members<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                int(smem));
     if (e != cudaSuccess) return e;
@@ -329,7 +329,7 @@ cudaError_t launch_gather_rows(const PatternDev& g, const WaveDev& w, int nb_max
                                double mu, double* A, NsStateDev ns, int* flags, cudaStream_t st) {
   if (w.nsub <= 0) return cudaSuccess;
   const size_t smem = size_t(nb_max) * 8 + size_t(2 * nb_max + 1) * 4 + size_t(ld_max) * 4;
-  if (smem > 48 * 1024) {
+  if (smem > kSmemByDefault) {
     const cudaError_t e = cudaFuncSetAttribute(k_gather_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
   }
@@ -363,7 +363,7 @@ cudaError_t launch_scatter_staged(const PatternDev& g, const WaveDev& w, NsState
   if (w.nsub <= 0) return cudaSuccess;
   const int chunk = scatter_chunk(ld_max, bs_max);
   const size_t smem = scatter_staged_smem(nb_max, ld_max, bs_max);
-  if (smem > 48 * 1024) {
+  if (smem > kSmemByDefault) {
     const cudaError_t e = cudaFuncSetAttribute(k_scatter_staged<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                int(smem));
     if (e != cudaSuccess) return e;

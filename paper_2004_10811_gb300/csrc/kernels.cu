@@ -412,7 +412,7 @@ template <typename T>
 static cudaError_t power_impl(const WaveDev& w, const T* X, int iters, const int* state, double* rho,
                               int max_ld, cudaStream_t st) {
   const size_t smem = size_t(2 * max_ld) * sizeof(float);
-  if (smem > 48 * 1024) {
+  if (smem > kSmemByDefault) {
     cudaError_t e = cudaFuncSetAttribute(k_power<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
   }
@@ -493,7 +493,7 @@ cudaError_t launch_gather(const PatternDev& g, const WaveDev& w, const int2* ite
   if (gather_rows_fits(nb_max, ld_max, bs_max))
     return launch_gather_rows(g, w, nb_max, ld_max, K, mu, A, ns, flags, st);
   const size_t smem = size_t(ld_max) * (sizeof(long long) + sizeof(int)) + size_t(3 * nb_max + 1) * sizeof(int);
-  if (smem > 48 * 1024) {
+  if (smem > kSmemByDefault) {
     cudaError_t e = cudaFuncSetAttribute(k_gather, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          int(smem));
     if (e != cudaSuccess) return e;
@@ -553,7 +553,7 @@ static cudaError_t scatter_impl(const PatternDev& g, const WaveDev& w, NsStateDe
                                     corr_a, corr_b, fallback, sqpart);
   const int nb_max = geo.nb_max;
   const size_t smem = size_t(nb_max + 1) * sizeof(int);
-  if (smem > 48 * 1024) {
+  if (smem > kSmemByDefault) {
     cudaError_t e = cudaFuncSetAttribute(k_scatter<T>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
